@@ -19,16 +19,18 @@
 //      same test in one lane.  For a sliding router (Sec. 5.2) a line word
 //      is the union of the slice bits not yet committed and the 32 stamps of
 //      the word that are active at the router's slice clock.
-//   Survivors are appended as (ip << 32 | z0) keys with one atomic per hit.
+//   Survivors are collected per warp and appended as (ip << 32 | z0) keys, up
+//   to 32 and more per atomic on the one result counter.
 // k_sort_emit: sorts the keys by ip (ascending; ips are unique) and writes
 //   sp_candidate records with est taken from a table of -k ln(z0 / k).  Up to
-//   8,192 keys one block sorts them in shared memory (bitonic).  Above that,
-//   the cooperative grid sorts runs of 8,192 keys in shared memory, one block
-//   per run, then merges pairs of runs in log2(runs) rounds between grid-wide
+//   2,048 keys one block sorts them in shared memory (bitonic).  Above that,
+//   the cooperative grid sorts runs of 2,048 keys in shared memory, one block
+//   per run, then merges groups of 16 runs per round between grid-wide
 //   barriers: each key's place in the merged run is its index in its own run
-//   plus the number of keys of the sibling run below it (binary search).
-//   The rounds alternate between the key buffer and the record buffer (which
-//   holds at least as many bytes), ending in the key buffer.
+//   plus the number of keys of the other 15 runs below it (binary searches
+//   side by side).  The rounds alternate between the key buffer and the record
+//   buffer (which holds at least as many bytes); the last one reads the key
+//   buffer and writes the records.
 #include <cooperative_groups.h>
 
 #include "sp_internal.h"
@@ -43,10 +45,12 @@ constexpr int kDetectWarps = 8;
 constexpr int kDetectThreads = kDetectWarps * 32;
 constexpr int kHostQueue = 256;                  // complete tuples queued per warp
 constexpr uint32_t kFull = 0xFFFFFFFFu;
-// SEAs of 512 bytes (profiles D, D3 and S) are staged in shared memory: a
-// ring of kSeaRing SEAs per warp, filled kSeaRing - 1 SEAs ahead of use
-constexpr uint32_t kStagedSea = 512;
-constexpr int kSeaRing = 4;
+constexpr int kPending = 64;                     // found keys a warp holds back before it appends them
+// SEAs of a multiple of 16 bytes, up to 1 KiB, are staged in shared memory: a
+// ring of 4 SEAs per warp (3 above 512 bytes, so that four blocks still share
+// an SM), filled one SEA less than the ring ahead of use
+constexpr uint32_t kStagedSea = 1024;
+constexpr int sea_ring(uint32_t sea_bytes) { return sea_bytes <= 512 ? 4 : 3; }
 
 // 16-byte asynchronous copy from global to shared memory (one per lane)
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
@@ -150,13 +154,37 @@ __device__ __forceinline__ bool emit_lp(const DevParams& d, const LdcaRead& ldca
   return true;
 }
 
+// Found keys of one warp, held back in shared memory (n is warp-uniform).  One
+// atomic per found host on the one result counter serialises in its L2 slice:
+// 150,000 results took 378 us that way; appended 32 and more at a time the
+// counter is out of the way.
+struct Pending {
+  uint64_t* keys;                                  // [kPending], shared memory
+  uint32_t n;
+};
+
+// appends the warp's pending keys (all lanes call it)
+__device__ __forceinline__ void flush_pending(Pending& p, const Found& f, uint32_t lane) {
+  if (p.n == 0) return;
+  __syncwarp();                                    // the keys are written
+  uint32_t at = 0;
+  if (lane == 0) at = atomicAdd(&f.status->count, p.n);
+  at = __shfl_sync(kFull, at, 0);
+  for (uint32_t i = lane; i < p.n; i += 32) {
+    if (at + i < f.cap) f.keys[at + i] = p.keys[i];
+    else atomicOr(&f.status->overflow, 1u);
+  }
+  p.n = 0;
+  __syncwarp();                                    // the keys are read
+}
+
 // The warp's LDCA test of n queued hosts (all lanes call it).  A host's LR
 // lines of wpl words are split over the lanes: with wpl >= 32 each lane
 // takes every 32nd word of each line and two hosts go per pass; with
 // wpl < 32 a pass takes 32 / wpl hosts, one word per lane.
 template <bool kSliding>
 __device__ void test_queue(const DevParams& d, const LdcaRead& ldca, const uint32_t* queue,
-                           uint32_t n, uint32_t z_theta, const Found& f, uint32_t lane) {
+                           uint32_t n, uint32_t z_theta, const Found& f, Pending& pend, uint32_t lane) {
   const uint32_t wpl = 1u << (d.k_log2 - 5u);
   const uint32_t k = 1u << d.k_log2;
   if (wpl >= 32) {
@@ -178,10 +206,13 @@ __device__ void test_queue(const DevParams& d, const LdcaRead& ldca, const uint3
         ones0 += __shfl_xor_sync(kFull, ones0, o);
         ones1 += __shfl_xor_sync(kFull, ones1, o);
       }
+      const bool keep0 = k - ones0 <= z_theta, keep1 = two && k - ones1 <= z_theta;   // warp-uniform
       if (lane == 0) {
-        keep_host(ip0, k - ones0, z_theta, f);
-        if (two) keep_host(ip1, k - ones1, z_theta, f);
+        if (keep0) pend.keys[pend.n] = ((uint64_t)ip0 << 32) | (k - ones0);
+        if (keep1) pend.keys[pend.n + (keep0 ? 1u : 0u)] = ((uint64_t)ip1 << 32) | (k - ones1);
       }
+      pend.n += (keep0 ? 1u : 0u) + (keep1 ? 1u : 0u);
+      if (pend.n > (uint32_t)kPending - 32u) flush_pending(pend, f, lane);
     }
   } else {
     const uint32_t per = 32u / wpl;                 // hosts per pass
@@ -196,37 +227,46 @@ __device__ void test_queue(const DevParams& d, const LdcaRead& ldca, const uint3
         ones = __popc(u);
       }
       for (uint32_t o = wpl >> 1; o > 0; o >>= 1) ones += __shfl_xor_sync(kFull, ones, o);
-      if (w == 0 && q < n) keep_host(queue[q], k - ones, z_theta, f);
+      const bool keep = w == 0 && q < n && k - ones <= z_theta;      // at most 32 hosts a pass
+      const uint32_t bal = __ballot_sync(kFull, keep);
+      if (keep) pend.keys[pend.n + __popc(bal & ((1u << lane) - 1u))] = ((uint64_t)queue[q] << 32) | (k - ones);
+      pend.n += __popc(bal);
+      if (pend.n > (uint32_t)kPending - 32u) flush_pending(pend, f, lane);
     }
   }
 }
 
-template <bool kSliding>
+template <bool kSliding, int kSeaRing>             // kSeaRing: SEAs per warp staged in shared memory, 0 = none
 __global__ void __launch_bounds__(kDetectThreads, 4)
 k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uint64_t* __restrict__ clock,
-         uint32_t k_slices, uint32_t z_theta, Found f, bool staged) {
+         uint32_t k_slices, uint32_t z_theta, Found f) {
+  constexpr bool staged = kSeaRing > 0;
   extern __shared__ __align__(16) uint32_t s_dyn[];
   if (kSliding) {                                   // the window of the router's current slice
     ldca.cur4 = ((uint32_t)(*clock % 255u) + 1u) * 0x01010101u;
     ldca.k4 = k_slices * 0x01010101u;
   }
   __shared__ uint32_t s_queue_n[kDetectWarps];
+  __shared__ uint64_t s_pending[kDetectWarps][kPending];
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   uint32_t* queue = s_dyn + warp * kHostQueue;           // [kDetectWarps][kHostQueue] IPs
   uint32_t* queue_n = &s_queue_n[warp];
   uint16_t* lists = reinterpret_cast<uint16_t*>(s_dyn + kDetectWarps * kHostQueue) + warp * d.sea_bytes;
+  Pending pend{s_pending[warp], 0u};
   if (lane == 0) *queue_n = 0;
   __syncwarp();
   const uint32_t n_sea = 1u << d.r;
   const uint32_t stride = gridDim.x * kDetectWarps;
-  // staged SEAs (512 bytes, 16-byte aligned SEAV): the warp's ring of
-  // kSeaRing SEAs after the lists; 16 bytes per lane and SEA by cp.async,
+  // staged SEAs (16-byte aligned SEAV and SEA size): the warp's ring of
+  // kSeaRing SEAs after the lists; 16 bytes per lane and copy by cp.async,
   // one commit group per SEA (empty past the last SEA, so that the count of
   // groups in flight stays fixed)
   uint8_t* ring = reinterpret_cast<uint8_t*>(s_dyn + kDetectWarps * kHostQueue) +
-                  (size_t)kDetectWarps * d.sea_bytes * sizeof(uint16_t) + (size_t)warp * kSeaRing * kStagedSea;
+                  (size_t)kDetectWarps * d.sea_bytes * sizeof(uint16_t) + (size_t)warp * kSeaRing * d.sea_bytes;
   auto stage_sea = [&](uint32_t rp, uint32_t slot) {
-    if (rp < n_sea) cp_async16(ring + slot * kStagedSea + 16u * lane, seav + (uint64_t)rp * kStagedSea + 16u * lane);
+    if (rp < n_sea)
+      for (uint32_t o = 16u * lane; o < d.sea_bytes; o += 512u)
+        cp_async16(ring + slot * d.sea_bytes + o, seav + (uint64_t)rp * d.sea_bytes + o);
     cp_async_commit();
   };
   uint32_t rp = blockIdx.x * kDetectWarps + warp;
@@ -246,10 +286,11 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
       // the SEA kSeaRing - 1 ahead goes to the slot this warp read last
       // (every lane passed the __syncwarp at the end of that iteration); then
       // wait for this SEA's copy and make every lane's bytes visible
-      stage_sea(rp + (uint32_t)(kSeaRing - 1) * stride, (it + kSeaRing - 1) % kSeaRing);
-      cp_async_wait<kSeaRing - 1>();
+      constexpr uint32_t R = staged ? kSeaRing : 1;
+      stage_sea(rp + (R - 1) * stride, (it + R - 1) % R);
+      cp_async_wait<R - 1>();
       __syncwarp();
-      sea = ring + (it % kSeaRing) * kStagedSea;
+      sea = ring + (it % R) * d.sea_bytes;
     }
     // 1. hot SEs per row
     uint32_t cnt[8];
@@ -341,20 +382,23 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
     __syncwarp();
     // 3. the warp's LDCA test of this SEA's complete tuples
     const uint32_t nq = min(*queue_n, (uint32_t)kHostQueue);
-    if (nq) test_queue<kSliding>(d, ldca, queue, nq, z_theta, f, lane);
+    if (nq) test_queue<kSliding>(d, ldca, queue, nq, z_theta, f, pend, lane);
     __syncwarp();
     if (lane == 0) *queue_n = 0;
     __syncwarp();
     const bool bound = (__shfl_sync(kFull, ov, 0) & 2u) != 0u;
     stop = __any_sync(kFull, stop) || bound;
   }
+  flush_pending(pend, f, lane);
   if (staged) cp_async_wait<0>();                  // no copy in flight at exit
-  if (join_local) atomicAdd(reinterpret_cast<unsigned long long*>(&f.status->join), (unsigned long long)join_local);
+  join_local = __reduce_add_sync(kFull, join_local);           // one atomic per warp
+  if (lane == 0 && join_local) atomicAdd(reinterpret_cast<unsigned long long*>(&f.status->join), (unsigned long long)join_local);
 }
 
 // ---- sort + emit ----------------------------------------------------------
 constexpr int kSortThreads = 1024;
-constexpr uint32_t kSmemSortCap = 8192;   // 64 KiB of keys
+constexpr uint32_t kRun = 2048;           // keys one block sorts in shared memory (16 KiB, two per thread)
+constexpr int kWays = 16;                 // runs merged per round
 
 __device__ __forceinline__ void emit_record(uint64_t key, const double* est_table, sp_candidate* out) {
   sp_candidate c;
@@ -366,123 +410,148 @@ __device__ __forceinline__ void emit_record(uint64_t key, const double* est_tabl
   *out = c;
 }
 
-// bitonic sort of m (a power of two, <= kSmemSortCap) keys in shared memory, ascending
+// bitonic sort of m (a power of two, 2 <= m <= kRun) keys in shared memory,
+// ascending; one compare-exchange per thread and stage.  A warp's 32
+// compare-exchanges of a stage with stride <= 32 stay within its own 64 keys,
+// so those stages need only the warp's own barrier.
 __device__ void smem_bitonic(uint64_t* a, uint32_t m) {
+  const uint32_t i = threadIdx.x;
   for (uint32_t size = 2; size <= m; size <<= 1) {
     for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
-      for (uint32_t i = threadIdx.x; i < m / 2; i += blockDim.x) {
+      if (i < m / 2) {
         const uint32_t lo = 2 * i - (i & (stride - 1));
         const uint32_t hi = lo + stride;
         const bool up = (lo & size) == 0;
         const uint64_t x = a[lo], y = a[hi];
         if ((x > y) == up) { a[lo] = y; a[hi] = x; }
       }
-      __syncthreads();
+      // the next stage's stride: stride / 2, or `size` at the start of the next size
+      const uint32_t next = stride > 1 ? stride >> 1 : size;
+      if (stride > 32u || next > 32u) __syncthreads();
+      else __syncwarp();
     }
   }
+  __syncthreads();
 }
 
-// number of keys of run[0, len) below key (the keys of a run are sorted and unique)
-__device__ __forceinline__ uint32_t count_below(const uint64_t* run, uint32_t len, uint64_t key) {
-  uint32_t lo = 0, hi = len;
-  while (lo < hi) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (run[mid] < key) lo = mid + 1;
-    else hi = mid;
+// Place of a key within its group of kWays runs of w keys (a power of two;
+// group = [base, end) of src, only its last run may be shorter): its index in
+// its own run plus the keys of every other run below it.  The searches of the
+// runs advance together, so a step costs one memory round trip for all.
+__device__ __forceinline__ uint32_t merged_place(const uint64_t* src, uint32_t base, uint32_t end, uint32_t w,
+                                                 uint32_t i, uint64_t key) {
+  const uint32_t own = (i - base) / w;
+  uint32_t pos[kWays];
+#pragma unroll
+  for (int q = 0; q < kWays; ++q) pos[q] = 0;
+  // after steps w, w / 2, ..., 1: pos[q] = keys of run q below key
+  for (uint32_t step = w; step > 0; step >>= 1) {
+#pragma unroll
+    for (int q = 0; q < kWays; ++q) {
+      const uint32_t at = pos[q] + step;                           // 1-based rank tried
+      const uint64_t g = (uint64_t)base + (uint64_t)q * w + at - 1;
+      if (at <= w && g < end && (uint32_t)q != own && src[g] < key) pos[q] = at;
+    }
   }
-  return lo;
+  uint32_t place = i - own * w;                                    // base + index in the own run
+#pragma unroll
+  for (int q = 0; q < kWays; ++q) place += pos[q];
+  return place;
 }
 
+// Bounds: latency.  Up to kRun keys: 66 stages in one block (4.4 us at ~500
+// keys).  Above: one run per block, then ceil(log16(runs)) merge rounds.
 __global__ void __launch_bounds__(kSortThreads)
 k_sort_emit(uint64_t* keys, uint32_t cap, const DetectStatus* status, const double* est_table,
             sp_candidate* out) {
-  extern __shared__ uint64_t s_keys[];
+  __shared__ uint64_t s_keys[kRun];
   const uint32_t n = min(status->count, cap);        // the same for every block
   if (n == 0) return;
-  if (n <= kSmemSortCap) {                          // one block, in shared memory
+  const uint32_t tid = threadIdx.x;
+  if (n <= kRun) {                                  // one block, in shared memory
     if (blockIdx.x != 0) return;
-    uint32_t m = 1;
+    uint32_t m = 2;
     while (m < n) m <<= 1;
-    for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) s_keys[i] = i < n ? keys[i] : ~0ull;
+    for (uint32_t i = tid; i < m; i += kSortThreads) s_keys[i] = i < n ? keys[i] : ~0ull;
     __syncthreads();
     smem_bitonic(s_keys, m);
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) emit_record(s_keys[i], est_table, out + i);
+    for (uint32_t i = tid; i < n; i += kSortThreads) emit_record(s_keys[i], est_table, out + i);
     return;
   }
   cg::grid_group grid = cg::this_grid();
-  // 1. runs of kSmemSortCap keys, sorted in shared memory, written back in place
-  const uint32_t runs = (n + kSmemSortCap - 1) / kSmemSortCap;
-  for (uint32_t r = blockIdx.x; r < runs; r += gridDim.x) {
-    const uint32_t base = r * kSmemSortCap;
-    const uint32_t len = min(kSmemSortCap, n - base);
-    for (uint32_t i = threadIdx.x; i < kSmemSortCap; i += blockDim.x) s_keys[i] = i < len ? keys[base + i] : ~0ull;
-    __syncthreads();
-    smem_bitonic(s_keys, kSmemSortCap);
-    for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) keys[base + i] = s_keys[i];
-    __syncthreads();
-  }
-  // 2. merge rounds; an odd number of rounds starts with a copy so that the
-  // last round writes the key buffer
-  uint32_t rounds = 0;
-  for (uint64_t w = kSmemSortCap; w < n; w <<= 1) ++rounds;
   uint64_t* tmp = reinterpret_cast<uint64_t*>(out);  // cap records of 24 bytes hold n keys
-  uint64_t* src = keys;
-  uint64_t* dst = tmp;
-  const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint64_t gsize = (uint64_t)gridDim.x * blockDim.x;
-  grid.sync();
-  if (rounds & 1u) {
-    for (uint64_t i = gtid; i < n; i += gsize) tmp[i] = keys[i];
-    src = tmp;
-    dst = keys;
-    grid.sync();
+  uint32_t rounds = 0;
+  for (uint64_t w = kRun; w < n; w *= kWays) ++rounds;   // >= 1
+  // 1. sorted runs, written where an odd number of rounds ends up reading the key buffer
+  uint64_t* src = (rounds & 1u) ? keys : tmp;
+  uint64_t* dst = (rounds & 1u) ? tmp : keys;
+  const uint32_t runs = (n + kRun - 1) / kRun;
+  for (uint32_t r = blockIdx.x; r < runs; r += gridDim.x) {
+    const uint32_t base = r * kRun;
+    const uint32_t len = min(kRun, n - base);
+    for (uint32_t i = tid; i < kRun; i += kSortThreads) s_keys[i] = i < len ? keys[base + i] : ~0ull;
+    __syncthreads();
+    smem_bitonic(s_keys, kRun);
+    for (uint32_t i = tid; i < len; i += kSortThreads) src[base + i] = s_keys[i];
+    __syncthreads();
   }
-  for (uint64_t w = kSmemSortCap; w < n; w <<= 1) {
-    for (uint64_t i = gtid; i < n; i += gsize) {
-      const uint64_t base = i / (2 * w) * (2 * w);
-      const uint64_t mid = base + w < n ? base + w : n;
-      const uint64_t end = base + 2 * w < n ? base + 2 * w : n;
-      const uint64_t key = src[i];
-      uint64_t pos;
-      if (i < mid) pos = i + count_below(src + mid, (uint32_t)(end - mid), key);          // run A
-      else pos = (i - mid) + base + count_below(src + base, (uint32_t)(mid - base), key);  // run B
-      dst[pos] = key;
-    }
+  // 2. merge rounds; the last one reads the key buffer and writes the records
+  const uint64_t gtid = (uint64_t)blockIdx.x * kSortThreads + tid;
+  const uint64_t gsize = (uint64_t)gridDim.x * kSortThreads;
+  for (uint64_t w = kRun; w < n; w *= kWays) {
     grid.sync();
+    const uint64_t group = w * kWays;
+    const bool last = group >= n;
+    for (uint64_t i = gtid; i < n; i += gsize) {
+      const uint64_t base = i / group * group;
+      const uint64_t end = base + group < n ? base + group : n;
+      const uint64_t key = src[i];
+      const uint32_t place = merged_place(src, (uint32_t)base, (uint32_t)end, (uint32_t)w, (uint32_t)i, key);
+      if (last) emit_record(key, est_table, out + place);
+      else dst[place] = key;
+    }
     uint64_t* t = src;
     src = dst;
     dst = t;
   }
-  // 3. records (src is the key buffer now)
-  for (uint64_t i = gtid; i < n; i += gsize) emit_record(src[i], est_table, out + i);
 }
 
 }  // namespace
 
 namespace {
 
-template <bool kSliding>
-cudaError_t detect_launch(const DevParams& d, const uint8_t* seav, const LdcaRead& ldca, const uint64_t* clock,
-                          uint32_t k_slices, uint32_t z_theta, uint64_t* keys, uint32_t cap, uint64_t max_join,
-                          DetectStatus* status, cudaStream_t s) {
-  // 512-byte SEAs of a 16-byte aligned SEAV are staged in shared memory
-  const bool staged = d.sea_bytes == kStagedSea && ((uintptr_t)seav & 15u) == 0u;
+template <bool kSliding, int kSeaRing>
+cudaError_t detect_launch_ring(const DevParams& d, const uint8_t* seav, const LdcaRead& ldca, const uint64_t* clock,
+                               uint32_t k_slices, uint32_t z_theta, const Found& f, cudaStream_t s) {
   const size_t smem = (size_t)kDetectWarps * kHostQueue * sizeof(uint32_t) +
                       (size_t)kDetectWarps * d.sea_bytes * sizeof(uint16_t) +
-                      (staged ? (size_t)kDetectWarps * kSeaRing * kStagedSea : 0u);
-  cudaError_t e = cudaFuncSetAttribute(k_detect<kSliding>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                      (size_t)kDetectWarps * kSeaRing * d.sea_bytes;
+  auto kern = k_detect<kSliding, kSeaRing>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_detect<kSliding>, kDetectThreads, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kDetectThreads, smem);
   if (per_sm < 1) per_sm = 1;
   const uint64_t n_sea = 1ull << d.r;
   uint64_t grid = (n_sea + kDetectWarps - 1) / kDetectWarps;
   if (grid > (uint64_t)sms * per_sm) grid = (uint64_t)sms * per_sm;
-  Found f{keys, cap, max_join, status};
-  k_detect<kSliding><<<(unsigned)grid, kDetectThreads, smem, s>>>(d, seav, ldca, clock, k_slices, z_theta, f, staged);
+  kern<<<(unsigned)grid, kDetectThreads, smem, s>>>(d, seav, ldca, clock, k_slices, z_theta, f);
   return cudaGetLastError();
+}
+
+template <bool kSliding>
+cudaError_t detect_launch(const DevParams& d, const uint8_t* seav, const LdcaRead& ldca, const uint64_t* clock,
+                          uint32_t k_slices, uint32_t z_theta, uint64_t* keys, uint32_t cap, uint64_t max_join,
+                          DetectStatus* status, cudaStream_t s) {
+  const Found f{keys, cap, max_join, status};
+  // staged SEAs need 16-byte copies; above kStagedSea a ring would cost blocks
+  if ((d.sea_bytes & 15u) != 0u || d.sea_bytes > kStagedSea || ((uintptr_t)seav & 15u) != 0u)
+    return detect_launch_ring<kSliding, 0>(d, seav, ldca, clock, k_slices, z_theta, f, s);
+  if (sea_ring(d.sea_bytes) == 4)
+    return detect_launch_ring<kSliding, 4>(d, seav, ldca, clock, k_slices, z_theta, f, s);
+  return detect_launch_ring<kSliding, 3>(d, seav, ldca, clock, k_slices, z_theta, f, s);
 }
 
 }  // namespace
@@ -505,21 +574,18 @@ cudaError_t launch_detect_sliding(const DevParams& d, const uint8_t* seav, const
 cudaError_t launch_sort_emit(uint64_t* keys, uint32_t cap, const DetectStatus* status,
                              const double* est_table, uint32_t /*k_log2*/,
                              sp_candidate* out, cudaStream_t s) {
-  const size_t smem = kSmemSortCap * sizeof(uint64_t);
-  cudaError_t e = cudaFuncSetAttribute(k_sort_emit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   // a cooperative grid (every block resident) of at most one block per SM,
   // and no more blocks than runs of the largest count
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sort_emit, kSortThreads, smem);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sort_emit, kSortThreads, 0);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const uint32_t max_runs = (cap + kSmemSortCap - 1) / kSmemSortCap;
+  const uint32_t max_runs = (cap + kRun - 1) / kRun;
   const unsigned grid = (unsigned)(max_runs < (uint32_t)sms ? (max_runs ? max_runs : 1u) : (uint32_t)sms);
   void* args[] = {&keys, &cap, &status, &est_table, &out};
-  e = cudaLaunchCooperativeKernel((const void*)k_sort_emit, dim3(grid), dim3(kSortThreads), args, smem, s);
+  e = cudaLaunchCooperativeKernel((const void*)k_sort_emit, dim3(grid), dim3(kSortThreads), args, 0, s);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
