@@ -118,6 +118,10 @@ struct sp_ctx {
   // list, which sets the device flag ovf[r] (cleared with the zeroing)
   bool* ldca_zero = nullptr;
   uint32_t* ovf = nullptr;
+  // set once a call of this context was recorded in a stream capture: a
+  // replay writes LDCAs that the host then knows nothing of, so ldca_zero says
+  // nothing any more
+  bool captured = false;
   // sliding window (Sec. 5): one stamp byte per bit, per-router slice clock;
   // the bit sketch of a sliding router holds the current slice's bits until
   // they are committed to the stamps
@@ -485,10 +489,28 @@ int sp_get_params(const sp_ctx* ctx, sp_params* out) {
   return SP_OK;
 }
 
+static bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    cudaGetLastError();                          // the legacy stream beside another thread's capture
+    return false;
+  }
+  return cs != cudaStreamCaptureStatusNone;
+}
+
+// Called first by every entry point that writes a sketch.
+static void note_capture(sp_ctx* ctx) {
+  if (!ctx->captured && capturing(ctx->stream)) ctx->captured = true;
+}
+
+// Whether a router's LDCA is known to be all zero but for spilled bits, which
+// its flag ovf[router] announces.
+static bool ldca_known_zero(const sp_ctx* ctx, uint32_t router) { return ctx->ldca_zero[router] && !ctx->captured; }
+
 // Folds a router's pending binned-scan planes into its LDCA.
 static int fold_router(sp_ctx* ctx, uint32_t router) {
   if (!ctx->planes_dirty[router]) return SP_OK;
-  const uint32_t* fresh = ctx->ldca_zero[router] ? ctx->ovf + router : nullptr;
+  const uint32_t* fresh = ldca_known_zero(ctx, router) ? ctx->ovf + router : nullptr;
   if (sp::launch_fold(ctx->d, ctx->planes[router], ctx->ldca(router), ctx->bs.fold_grid, ctx->stream, fresh) !=
       cudaSuccess)
     return SP_ERR_CUDA;
@@ -620,19 +642,44 @@ static int commit_seav_window(sp_ctx* ctx, uint32_t router) {
   return SP_OK;
 }
 
+// Zeroes routers first .. first + count - 1 of a discrete context.  An LDCA
+// that only binned rounds could have written and that was never folded is
+// still all zero unless its flag says otherwise: a step that merges its
+// routers' planes (sp_merge) never writes their LDCAs, and zeroing the 16 of
+// profile D3 again took 250 of 446 us.  Without such a router
+// one plain launch zeroes sketches and flags.
+static int zero_routers(sp_ctx* ctx, uint32_t first, uint32_t count) {
+  sp::RouterSet clean{};
+  bool any = false;
+  for (uint32_t r = first; r < first + count; ++r)
+    if (ldca_known_zero(ctx, r)) {
+      clean.w[r >> 5] |= 1u << (r & 31u);
+      any = true;
+    }
+  const cudaError_t e =
+      any ? sp::launch_reset(ctx->sketches, ctx->stride, ctx->seav_pad, first, count, clean, ctx->ovf, ctx->stream)
+          : sp::launch_zero_flags(ctx->seav(first), ctx->stride * count, ctx->ovf + first, count, ctx->stream);
+  if (e != cudaSuccess) return SP_ERR_CUDA;
+  for (uint32_t r = first; r < first + count; ++r) {
+    ctx->planes_dirty[r] = false;                // pending planes belong to the old window
+    ctx->slice_dirty[r] = false;
+    ctx->ldca_zero[r] = true;
+  }
+  return SP_OK;
+}
+
 int sp_reset(sp_ctx* ctx, uint32_t router) {
   if (!ctx) return SP_ERR_PARAM;
   if (router >= ctx->p.n_routers) return SP_ERR_ROUTER;
+  note_capture(ctx);
+  if (!ctx->sliding) return zero_routers(ctx, router, 1);
   ctx->planes_dirty[router] = false;     // pending planes belong to the old window
   ctx->slice_dirty[router] = false;
-  if (ctx->sliding) {
-    ctx->slice[router] = 0;
-    if (cudaMemsetAsync(ctx->dev_clock(router), 0, sizeof(uint64_t), ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
-    if (sp::launch_zero(ctx->st_seav(router), ctx->st_stride, ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
-  }
+  ctx->slice[router] = 0;
+  if (cudaMemsetAsync(ctx->dev_clock(router), 0, sizeof(uint64_t), ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
+  if (sp::launch_zero(ctx->st_seav(router), ctx->st_stride, ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
   if (sp::launch_zero_flags(ctx->seav(router), ctx->stride, ctx->ovf + router, 1, ctx->stream) != cudaSuccess)
     return SP_ERR_CUDA;
-  ctx->ldca_zero[router] = !ctx->sliding;
   return SP_OK;
 }
 
@@ -640,21 +687,12 @@ int sp_reset_range(sp_ctx* ctx, uint32_t first, uint32_t count) {
   if (!ctx) return SP_ERR_PARAM;
   if (count == 0) return SP_OK;
   if (first >= ctx->p.n_routers || count > ctx->p.n_routers - first) return SP_ERR_ROUTER;
-  if (ctx->sliding) {                            // stamps and clocks are per router
-    for (uint32_t r = first; r < first + count; ++r) {
-      const int rc = sp_reset(ctx, r);
-      if (rc != SP_OK) return rc;
-    }
-    return SP_OK;
-  }
-  // the routers' regions are contiguous: one zeroing launch for all of them
-  if (sp::launch_zero_flags(ctx->seav(first), ctx->stride * count, ctx->ovf + first, count, ctx->stream) !=
-      cudaSuccess)
-    return SP_ERR_CUDA;
-  for (uint32_t r = first; r < first + count; ++r) {
-    ctx->planes_dirty[r] = false;                // pending planes belong to the old window
-    ctx->slice_dirty[r] = false;
-    ctx->ldca_zero[r] = true;
+  note_capture(ctx);
+  // discrete: the routers' regions are contiguous, one zeroing launch for all of them
+  if (!ctx->sliding) return zero_routers(ctx, first, count);
+  for (uint32_t r = first; r < first + count; ++r) {          // stamps and clocks are per router
+    const int rc = sp_reset(ctx, r);
+    if (rc != SP_OK) return rc;
   }
   return SP_OK;
 }
@@ -664,6 +702,7 @@ int sp_update(sp_ctx* ctx, uint32_t router, const uint32_t* dev_pairs, uint64_t 
   if (router >= ctx->p.n_routers) return SP_ERR_ROUTER;
   if (n_pairs == 0) return SP_OK;
   if (!dev_pairs || ((uintptr_t)dev_pairs & 7u)) return SP_ERR_PARAM;
+  note_capture(ctx);
   return do_update(ctx, router, dev_pairs, n_pairs);
 }
 
@@ -683,6 +722,7 @@ int sp_update_host(sp_ctx* ctx, uint32_t router, const uint32_t* host_pairs, uin
   if (router >= ctx->p.n_routers) return SP_ERR_ROUTER;
   if (n_pairs == 0) return SP_OK;
   if (!host_pairs) return SP_ERR_PARAM;
+  note_capture(ctx);
   int rc = ensure_staging(ctx);
   if (rc != SP_OK) return rc;
   const bool binned = use_binned(ctx, n_pairs);
@@ -730,11 +770,6 @@ int sp_update_host(sp_ctx* ctx, uint32_t router, const uint32_t* host_pairs, uin
     done += round_n;
   }
   return SP_OK;
-}
-
-static bool capturing(cudaStream_t st) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
 }
 
 // Uploads n entries of a batch table through the next pinned slot of the
@@ -925,6 +960,7 @@ int sp_update_batched_device(sp_ctx* ctx, const sp_batch* dev_batches, uint32_t 
   if (!ctx) return SP_ERR_PARAM;
   if (n_batches == 0) return SP_OK;
   if (!dev_batches || n_batches > 8192) return SP_ERR_PARAM;
+  note_capture(ctx);
   // the table is read on the device: any router may receive bits
   for (uint32_t r = 0; r < ctx->p.n_routers; ++r) {
     ctx->slice_dirty[r] = true;
@@ -1053,7 +1089,7 @@ int sp_merge(sp_ctx* ctx, const uint32_t* routers, uint32_t n, uint32_t dst_rout
   if (dst_router >= ctx->p.n_routers) return SP_ERR_ROUTER;
   for (uint32_t i = 0; i < n; ++i)
     if (routers[i] >= ctx->p.n_routers) return SP_ERR_ROUTER;
-  ctx->ldca_zero[dst_router] = false;
+  note_capture(ctx);
   std::vector<const uint8_t*> srcs;                // every listed router but dst (x | x = x)
   srcs.reserve(n);
   if (ctx->sliding) {
@@ -1068,15 +1104,42 @@ int sp_merge(sp_ctx* ctx, const uint32_t* routers, uint32_t n, uint32_t dst_rout
     return sp::launch_merge_stamp(ctx->st_seav(dst_router), srcs.data(), (uint32_t)srcs.size(), ctx->st_stride,
                                   ctx->dev_clock(dst_router), ctx->stream) == cudaSuccess ? SP_OK : SP_ERR_CUDA;
   }
-  int rc = fold_router(ctx, dst_router);
-  if (rc != SP_OK) return rc;
+  // Pending planes of the sources (and of dst) are folded straight into dst's
+  // LDCA, all of them in one pass: the sources keep theirs pending, and an
+  // LDCA that is known to be zero is not read.  Without pending planes the
+  // whole sketches are ORed by one plain pass.
+  bool pending = ctx->planes_dirty[dst_router];
+  std::vector<sp::FoldSrc> folds;
+  folds.reserve(n + 1);
+  if (pending) folds.push_back(sp::FoldSrc{ctx->planes[dst_router], nullptr, nullptr});
   for (uint32_t i = 0; i < n; ++i) {
-    rc = fold_router(ctx, routers[i]);
-    if (rc != SP_OK) return rc;
-    if (routers[i] != dst_router) srcs.push_back(ctx->seav(routers[i]));
+    const uint32_t r = routers[i];
+    if (r == dst_router) continue;
+    srcs.push_back(ctx->seav(r));
+    const bool dirty = ctx->planes_dirty[r];
+    pending = pending || dirty;
+    folds.push_back(sp::FoldSrc{dirty ? ctx->planes[r] : nullptr, ctx->ldca(r),
+                                ldca_known_zero(ctx, r) ? ctx->ovf + r : nullptr});
   }
-  return sp::launch_merge(ctx->seav(dst_router), srcs.data(), (uint32_t)srcs.size(), ctx->stride, ctx->stream) ==
-                 cudaSuccess ? SP_OK : SP_ERR_CUDA;
+  if (srcs.empty()) return fold_router(ctx, dst_router);
+  const uint32_t* fresh = ldca_known_zero(ctx, dst_router) ? ctx->ovf + dst_router : nullptr;
+  ctx->ldca_zero[dst_router] = false;
+  if (!pending)
+    return sp::launch_merge(ctx->seav(dst_router), srcs.data(), (uint32_t)srcs.size(), ctx->stride, ctx->stream) ==
+                   cudaSuccess ? SP_OK : SP_ERR_CUDA;
+  if (sp::launch_merge(ctx->seav(dst_router), srcs.data(), (uint32_t)srcs.size(), ctx->seav_pad, ctx->stream) !=
+      cudaSuccess) return SP_ERR_CUDA;
+  for (size_t base = 0; base < folds.size(); base += sp::kFoldMaxSrc) {
+    sp::FoldSrcs l{};
+    while (l.count < (uint32_t)sp::kFoldMaxSrc && base + l.count < folds.size()) {
+      l.s[l.count] = folds[base + l.count];
+      ++l.count;
+    }
+    if (sp::launch_fold_multi(ctx->d, l, ctx->ldca(dst_router), ctx->bs.fold_grid, ctx->stream,
+                              base == 0 ? fresh : nullptr) != cudaSuccess) return SP_ERR_CUDA;
+  }
+  ctx->planes_dirty[dst_router] = false;
+  return SP_OK;
 }
 
 int sp_copy_sketch(sp_ctx* ctx, uint32_t router, void* dev_dst, uint64_t cap, uint64_t* n) {
@@ -1086,6 +1149,7 @@ int sp_copy_sketch(sp_ctx* ctx, uint32_t router, void* dev_dst, uint64_t cap, ui
   if (!dev_dst) return SP_OK;
   if (cap < ctx->stride) return SP_ERR_TRUNCATED;
   if ((uintptr_t)dev_dst & 15u) return SP_ERR_PARAM;
+  note_capture(ctx);
   int frc = ctx->sliding ? commit_window(ctx, router) : fold_router(ctx, router);
   if (frc != SP_OK) return frc;
   const uint8_t* src = ctx->sliding ? ctx->wseav(router) : ctx->seav(router);
@@ -1097,6 +1161,7 @@ int sp_merge_device(sp_ctx* ctx, const void* const* dev_images, uint32_t n, uint
   if (!ctx || (n && !dev_images)) return SP_ERR_PARAM;
   if (dst_router >= ctx->p.n_routers) return SP_ERR_ROUTER;
   if (ctx->sliding) return SP_ERR_STATE;      // an image holds window bits, not slice stamps
+  note_capture(ctx);
   std::vector<const uint8_t*> srcs(n);
   for (uint32_t i = 0; i < n; ++i) {
     if (!dev_images[i] || ((uintptr_t)dev_images[i] & 15u)) return SP_ERR_PARAM;
@@ -1112,6 +1177,7 @@ int sp_merge_device(sp_ctx* ctx, const void* const* dev_images, uint32_t n, uint
 int sp_detect_async(sp_ctx* ctx, uint32_t router, uint32_t threshold) {
   if (!ctx) return SP_ERR_PARAM;
   if (router >= ctx->p.n_routers) return SP_ERR_ROUTER;
+  note_capture(ctx);
   if (threshold == 0) threshold = ctx->p.theta;
   const uint32_t zt = sp_z_theta(ctx->p.k_log2, threshold);
   int frc = ctx->sliding ? commit_seav_window(ctx, router) : fold_router(ctx, router);
@@ -1209,6 +1275,7 @@ int sp_results_device(sp_ctx* ctx, const sp_candidate** dev_records, const uint3
 int sp_slide(sp_ctx* ctx, uint32_t router) {
   if (!ctx) return SP_ERR_PARAM;
   if (router >= ctx->p.n_routers) return SP_ERR_ROUTER;
+  note_capture(ctx);
   if (!ctx->sliding) return sp_reset(ctx, router);   // discrete window: the next period starts empty
   int rc = commit(ctx, router);                       // slice t's bits carry id(t)
   if (rc != SP_OK) return rc;

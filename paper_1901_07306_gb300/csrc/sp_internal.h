@@ -96,6 +96,14 @@ struct BinnedScratch {
 cudaError_t launch_zero(void* dev, uint64_t bytes, cudaStream_t s);
 // launch_zero, and flags[0, n_flags) = 0 in the same launch
 cudaError_t launch_zero_flags(void* dev, uint64_t bytes, uint32_t* flags, uint32_t n_flags, cudaStream_t s);
+// A set of a context's routers (at most 4,096), as a kernel argument.
+struct RouterSet {
+  uint32_t w[128];
+};
+// Zeroes routers first .. first + count - 1 (sketches of `stride` bytes from
+// base) and their flags ovf; the LDCA of a router in `clean` only if its flag is set.
+cudaError_t launch_reset(uint8_t* base, uint64_t stride, uint64_t seav_pad, uint32_t first, uint32_t count,
+                         const RouterSet& clean, uint32_t* ovf, cudaStream_t s);
 cudaError_t launch_scan(const DevParams& d, uint8_t* seav, uint32_t* ldca,
                         const uint32_t* pairs, uint64_t n_pairs, int grid, cudaStream_t s);
 int scan_grid(const DevParams& d);
@@ -129,6 +137,23 @@ cudaError_t launch_scan_binned(const DevParams& d, uint8_t* seav, uint32_t* ldca
 // nullptr: ldca |= transpose(planes).
 cudaError_t launch_fold(const DevParams& d, const uint32_t* planes, uint32_t* ldca, int grid, cudaStream_t st,
                         const uint32_t* fresh = nullptr);
+// Up to kFoldMaxSrc routers folded into one LDCA: a router's pending planes
+// (null: none) and its LDCA, read unless null, or unless ovf is not null and
+// the flag it points at is 0 (the LDCA is still all zero then, see
+// BinnedScratch::ovf).
+constexpr int kFoldMaxSrc = 32;
+struct FoldSrc {
+  const uint32_t* planes;
+  const uint32_t* ldca;
+  const uint32_t* ovf;
+};
+struct FoldSrcs {
+  FoldSrc s[kFoldMaxSrc];
+  uint32_t count;
+};
+// ldca |= transpose(OR of the sources' planes) | OR of their LDCAs; fresh as in launch_fold
+cudaError_t launch_fold_multi(const DevParams& d, const FoldSrcs& src, uint32_t* ldca, int grid, cudaStream_t st,
+                              const uint32_t* fresh);
 // Sliding window stamps (Sec. 5.2): one byte per bit holding the id of the
 // last slice that set it, id(t) = t mod 255 + 1 (0 = never set).  Byte j of
 // active_mask4 is 0xFF iff byte j of s is an active stamp: non-zero, of age

@@ -2,6 +2,10 @@
 //
 // k_zero: every bit of SEAV and LDCA is 0 at the beginning of a time period
 //   (Sec. 3.1, Sec. 3.3).
+// k_reset: the same for a range of routers whose LDCAs may be known to be all
+//   zero already (written by nothing but binned rounds, whose bits wait in the
+//   plane accumulators): those are skipped unless the router's flag says that
+//   a bit bypassed the planes.
 // k_merge: the global server's SEAV/LDCA (Sec. 4.2) as the bitwise OR of the
 //   watch points' equal-size sketches; one pass reads every source once and
 //   writes the destination once (uint4, grid-stride, HBM bound).
@@ -24,6 +28,23 @@ k_zero(uint4* __restrict__ p, uint64_t n16, uint32_t* __restrict__ flags, uint32
   const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (uint64_t i = gid; i < n16; i += (uint64_t)gridDim.x * blockDim.x) p[i] = z;
   for (uint64_t i = gid; i < n_flags; i += (uint64_t)gridDim.x * blockDim.x) flags[i] = 0u;
+}
+
+// Routers first .. first + count - 1 of a context: the SEAV, and the LDCA
+// unless bit r of `clean` is set and ovf[r] is 0.  Every block takes its share
+// of every router (one that is zeroed whole among many skipped ones is spread
+// over the chip).  Blocks read all flags, so the caller clears them after the launch.
+__global__ void __launch_bounds__(kThreads)
+k_reset(uint8_t* __restrict__ base, uint64_t stride, uint64_t seav16, uint32_t first, uint32_t count,
+        RouterSet clean, const uint32_t* __restrict__ ovf) {
+  const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+  for (uint32_t r = first; r < first + count; ++r) {
+    const bool skip = ((clean.w[r >> 5] >> (r & 31u)) & 1u) != 0u && ovf[r] == 0u;
+    uint4* p = reinterpret_cast<uint4*>(base + (uint64_t)r * stride);
+    const uint64_t n16 = skip ? seav16 : stride / 16;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (uint64_t)gridDim.x * blockDim.x)
+      p[i] = z;
+  }
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -61,6 +82,16 @@ cudaError_t launch_zero_flags(void* dev, uint64_t bytes, uint32_t* flags, uint32
 
 cudaError_t launch_zero(void* dev, uint64_t bytes, cudaStream_t s) {
   return launch_zero_flags(dev, bytes, nullptr, 0u, s);
+}
+
+cudaError_t launch_reset(uint8_t* base, uint64_t stride, uint64_t seav_pad, uint32_t first, uint32_t count,
+                         const RouterSet& clean, uint32_t* ovf, cudaStream_t s) {
+  if (count == 0) return cudaSuccess;
+  uint64_t grid = (stride / 16 + kThreads - 1) / kThreads;
+  if (grid > (uint64_t)stream_grid()) grid = stream_grid();
+  k_reset<<<(unsigned)grid, kThreads, 0, s>>>(base, stride, seav_pad / 16, first, count, clean, ovf);
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : cudaMemsetAsync(ovf + first, 0, sizeof(uint32_t) * count, s);
 }
 
 cudaError_t launch_merge(uint8_t* dst, const uint8_t* const* srcs, uint32_t n_src,

@@ -449,15 +449,72 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, uint32_t lane) {
   return x;
 }
 
+// 256-bit load of 8 words (a 32-byte aligned plane chunk, one full sector).
+__device__ __forceinline__ void ld_chunk(const uint32_t* src, uint32_t (&v)[8]) {
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "l"(src));
+}
+
+// 32 x 32 bit transposes of 8 blocks, one per q = lane / 4: lane (q, s) holds
+// rows p = 4 i + s of block q in x[i] (bit c = column c) and afterwards columns
+// c = 4 i + s (bit p = row p's bit c).  Row bits 2 - 4 are register indices, so
+// three of the five butterfly stages stay in the lane (two byte permutes, one
+// shift and select); row bits 0 and 1 are lane bits: one shuffle, one
+// rotation and one select per word.
+__device__ __forceinline__ void transpose8x4(uint32_t (&x)[8], uint32_t lane) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {                      // rows p and p + 16
+    const uint32_t a = x[i], b = x[i + 4];
+    x[i] = __byte_perm(a, b, 0x5410);
+    x[i + 4] = __byte_perm(a, b, 0x7632);
+  }
+#pragma unroll
+  for (int h = 0; h < 8; h += 4) {
+#pragma unroll
+    for (int i = h; i < h + 2; ++i) {                // rows p and p + 8
+      const uint32_t a = x[i], b = x[i + 2];
+      x[i] = __byte_perm(a, b, 0x6240);
+      x[i + 2] = __byte_perm(a, b, 0x7351);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) {                   // rows p and p + 4
+    const uint32_t a = x[i], b = x[i + 1];
+    x[i] = (a & 0x0F0F0F0Fu) | ((b << 4) & 0xF0F0F0F0u);
+    x[i + 1] = ((a >> 4) & 0x0F0F0F0Fu) | (b & 0xF0F0F0F0u);
+  }
+  const bool hi2 = (lane & 2u) != 0u, hi1 = (lane & 1u) != 0u;
+  const uint32_t keep2 = hi2 ? 0xCCCCCCCCu : 0x33333333u, rot2 = hi2 ? 30u : 2u;
+  const uint32_t keep1 = hi1 ? 0xAAAAAAAAu : 0x55555555u, rot1 = hi1 ? 31u : 1u;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {                      // rows p and p + 2, then p and p + 1: across lanes
+    const uint32_t y = __shfl_xor_sync(kFull, x[i], 2);
+    x[i] = (x[i] & keep2) | (__funnelshift_l(y, y, rot2) & ~keep2);
+    const uint32_t z = __shfl_xor_sync(kFull, x[i], 1);
+    x[i] = (x[i] & keep1) | (__funnelshift_l(z, z, rot1) & ~keep1);
+  }
+}
+
+// The folds: ldca (= dst's) |= transpose(OR of the sources' planes) | OR of the
+// sources' LDCAs.  One source, the router itself, before a detect, export or
+// copy; the merge of Sec. 4.2 folds all watch points' pending planes at once
+// (16 routers of profile D3: one pass over 16 x 128 MiB of planes instead of 16
+// folds and a merge of 16 LDCAs, 1,668 -> 678 us).
 // planes: [ceil(W / 8)][k][8] words (W = LR * LC / 32 words per plane, 8-word
 // chunks of the k planes side by side); ldca: [LR * LC][k / 32] words.
-// A warp task is 8 consecutive plane words J0 .. J0 + 7 (one 32-byte chunk of
-// each plane it reads; 32 planes' chunks are 1 KiB of contiguous memory)
-// times 4 consecutive LDC words: it transposes 32 planes x 32 LDCs per word
-// and ORs the result into the lanes' LDC lines.
-__global__ void __launch_bounds__(256)
-k_fold(const uint32_t* __restrict__ planes, uint32_t* __restrict__ ldca, uint32_t W, uint32_t k_log2,
-       const uint32_t* __restrict__ fresh) {
+// A source's LDCA is read unless it is null or a flag beside it says that it is
+// still all zero (FoldSrc).
+__device__ __forceinline__ const uint32_t* live_ldca(const FoldSrc& s) {
+  return (s.ldca == nullptr || (s.ovf != nullptr && *s.ovf == 0u)) ? nullptr : s.ldca;
+}
+
+// k < 256.  A warp task is 8 consecutive plane words J0 .. J0 + 7 (one 32-byte
+// chunk of each plane it reads; 32 planes' chunks are 1 KiB of contiguous
+// memory) times 4 consecutive LDC words: it transposes 32 planes x 32 LDCs per
+// word and ORs the result into the lanes' LDC lines.
+__global__ void __launch_bounds__(256, 2)
+k_fold(FoldSrcs src, uint32_t* ldca, uint32_t W, uint32_t k_log2, const uint32_t* __restrict__ fresh) {
   const bool write_only = fresh != nullptr && *fresh == 0u;       // the LDCA is all zero: no read
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t wpl = 1u << (k_log2 - 5u);                       // words per LDC
@@ -469,45 +526,58 @@ k_fold(const uint32_t* __restrict__ planes, uint32_t* __restrict__ ldca, uint32_
     const uint64_t g = t / n_q;
     const uint32_t J0 = (uint32_t)(g * 8);
     const uint32_t nj = (W - J0) < 8u ? (W - J0) : 8u;
-    {
-      const uint32_t q0 = (uint32_t)(t % n_q) * 4u;
-      uint32_t x[4][8];
+    const uint32_t q0 = (uint32_t)(t % n_q) * 4u;
+    uint32_t x[4][8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) x[u][j] = 0u;
+    for (uint32_t s = 0; s < src.count; ++s) {
+      const uint32_t* planes = src.s[s].planes;
+      if (planes == nullptr) continue;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const uint32_t q = q0 + u;
         const uint32_t keep = q < wpl ? kFull : 0u;     // planes past k (k < 128 only) read as zero
-        const uint4* chunk = reinterpret_cast<const uint4*>(planes + g * ((uint64_t)wpl * 256u) +
-                                                            (uint64_t)((q < wpl ? q : 0u) * 32u + lane) * 8u);
-        const uint4 a = chunk[0], c = chunk[1];
-        x[u][0] = a.x & keep; x[u][1] = a.y & keep; x[u][2] = a.z & keep; x[u][3] = a.w & keep;
-        x[u][4] = c.x & keep; x[u][5] = c.y & keep; x[u][6] = c.z & keep; x[u][7] = c.w & keep;
+        uint32_t v[8];
+        ld_chunk(planes + g * ((uint64_t)wpl * 256u) + (uint64_t)((q < wpl ? q : 0u) * 32u + lane) * 8u, v);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[u][j] |= v[j] & keep;
       }
+    }
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if ((uint32_t)j >= nj) break;
-        uint32_t acc[4];
+    for (int j = 0; j < 8; ++j) {
+      if ((uint32_t)j >= nj) break;
+      uint32_t acc[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] = transpose32(x[u][j], lane);
-        uint32_t* line = ldca + ((uint64_t)(J0 + j) * 32u + lane) * wpl;
-        if (wpl >= 4) {
-          uint4 o = write_only ? make_uint4(0u, 0u, 0u, 0u) : *reinterpret_cast<uint4*>(line + q0);
-          o.x |= acc[0]; o.y |= acc[1]; o.z |= acc[2]; o.w |= acc[3];
-          *reinterpret_cast<uint4*>(line + q0) = o;
-        } else {
-          for (uint32_t u = 0; u < wpl; ++u) line[u] = (write_only ? 0u : line[u]) | acc[u];
+      for (int u = 0; u < 4; ++u) acc[u] = transpose32(x[u][j], lane);
+      const uint64_t at = ((uint64_t)(J0 + j) * 32u + lane) * wpl;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (q0 + u >= wpl) break;
+        uint32_t o = acc[u] | (write_only ? 0u : ldca[at + q0 + u]);
+        for (uint32_t s = 0; s < src.count; ++s) {
+          const uint32_t* l = live_ldca(src.s[s]);
+          if (l != nullptr) o |= l[at + q0 + u];
         }
+        ldca[at + q0 + u] = o;
       }
     }
   }
 }
 
 // k_fold8 (k >= 256): a warp task is 8 plane words J0 .. J0 + 7 times 8
-// consecutive LDC words q0 .. q0 + 7, so each lane ORs one whole 32-byte
-// sector into each of its 8 LDC lines; the 8 chunks of 8 planes' words are
-// loaded up front (16 loads in flight per lane).
-__global__ void __launch_bounds__(256)
-k_fold8(const uint32_t* __restrict__ planes, uint32_t* __restrict__ ldca, uint32_t W, uint32_t k_log2,
-        const uint32_t* __restrict__ fresh) {
+// consecutive LDC words q0 .. q0 + 7 (256 planes).  Lane (q, s) = (lane / 4,
+// lane mod 4) holds the chunks of planes 32 (q0 + q) + 4 i + s, i < 8: each of
+// its 8 loads takes a whole 32-byte sector per lane and whole 128-byte lines
+// per 4 lanes, and transpose8x4 leaves it word q0 + q of LDCs 32 J + 4 i + s,
+// so a store covers 4 whole sectors.  Bounds: the 2 x 32 MiB it moves at
+// profile D; with the 5-shuffle transpose per word and 16-byte accesses it
+// took 22 us there, this way 12.5 us.
+constexpr int kFold8Threads = 128;
+template <bool kMulti>
+__global__ void __launch_bounds__(kFold8Threads, kMulti ? 3 : 4)
+k_fold8(FoldSrcs src, uint32_t* ldca, uint32_t W, uint32_t k_log2, const uint32_t* __restrict__ fresh) {
   const bool write_only = fresh != nullptr && *fresh == 0u;       // the LDCA is all zero: no read
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t wpl = 1u << (k_log2 - 5u);                       // words per LDC, >= 8
@@ -515,35 +585,59 @@ k_fold8(const uint32_t* __restrict__ planes, uint32_t* __restrict__ ldca, uint32
   const uint64_t nwarp = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint64_t n_groups = (W + 7) / 8;
   const uint32_t n_q = wpl / 8;                                    // groups of 8 LDC words
+  const uint32_t q = lane >> 2, sub = lane & 3u;
+  bool any_ldca = false;                                          // some source's LDCA holds bits
+  if (kMulti)
+    for (uint32_t s = 0; s < src.count; ++s) any_ldca |= live_ldca(src.s[s]) != nullptr;
   for (uint64_t t = gwarp; t < n_groups * n_q; t += nwarp) {
     const uint64_t g = t / n_q;
     const uint32_t J0 = (uint32_t)(g * 8);
     const uint32_t nj = (W - J0) < 8u ? (W - J0) : 8u;
     const uint32_t q0 = (uint32_t)(t % n_q) * 8u;
-    uint32_t x[8][8];
+    const uint64_t chunk = g * ((uint64_t)wpl * 256u) + (uint64_t)((q0 + q) * 32u + sub) * 8u;
+    uint32_t x[8][8];                                              // [i][j]
+    if (!kMulti) {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const uint4* chunk = reinterpret_cast<const uint4*>(planes + g * ((uint64_t)wpl * 256u) +
-                                                          (uint64_t)((q0 + u) * 32u + lane) * 8u);
-      const uint4 a = chunk[0], c = chunk[1];
-      x[u][0] = a.x; x[u][1] = a.y; x[u][2] = a.z; x[u][3] = a.w;
-      x[u][4] = c.x; x[u][5] = c.y; x[u][6] = c.z; x[u][7] = c.w;
+      for (int i = 0; i < 8; ++i) ld_chunk(src.s[0].planes + chunk + i * 32, x[i]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[i][j] = 0u;
+      for (uint32_t s = 0; s < src.count; ++s) {
+        const uint32_t* planes = src.s[s].planes;
+        if (planes == nullptr) continue;
+        uint32_t v[8][8];                                          // 8 loads in flight beside the 64 sums
+#pragma unroll
+        for (int i = 0; i < 8; ++i) ld_chunk(planes + chunk + i * 32, v[i]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[i][j] |= v[i][j];
+      }
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       if ((uint32_t)j >= nj) break;
-      uint4* line = reinterpret_cast<uint4*>(ldca + ((uint64_t)(J0 + j) * 32u + lane) * wpl + q0);
-      uint4 o0 = make_uint4(0u, 0u, 0u, 0u), o1 = o0;
+      uint32_t w[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) w[i] = x[i][j];
+      transpose8x4(w, lane);
+      const uint64_t at = ((uint64_t)(J0 + j) * 32u + sub) * wpl + q0 + q;     // + 4 i LDCs
       if (!write_only) {
-        o0 = line[0];
-        o1 = line[1];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] |= ldca[at + (uint64_t)(4 * i) * wpl];
       }
-      o0.x |= transpose32(x[0][j], lane); o0.y |= transpose32(x[1][j], lane);
-      o0.z |= transpose32(x[2][j], lane); o0.w |= transpose32(x[3][j], lane);
-      o1.x |= transpose32(x[4][j], lane); o1.y |= transpose32(x[5][j], lane);
-      o1.z |= transpose32(x[6][j], lane); o1.w |= transpose32(x[7][j], lane);
-      line[0] = o0;
-      line[1] = o1;
+      if (kMulti && any_ldca) {
+        for (uint32_t s = 0; s < src.count; ++s) {
+          const uint32_t* l = live_ldca(src.s[s]);
+          if (l == nullptr) continue;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) w[i] |= l[at + (uint64_t)(4 * i) * wpl];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) ldca[at + (uint64_t)(4 * i) * wpl] = w[i];
     }
   }
 }
@@ -637,12 +731,22 @@ int binned_ctas(const BinShape& shape) { return sm_count() * (int)shape.per_sm; 
 
 int binned_fold_grid() { return sm_count() * 8; }
 
+cudaError_t launch_fold_multi(const DevParams& d, const FoldSrcs& src, uint32_t* ldca, int grid, cudaStream_t st,
+                              const uint32_t* fresh) {
+  const uint32_t words = (uint32_t)(((uint64_t)d.lr << d.lc_log2) >> 5);
+  if (d.k_log2 < 8) k_fold<<<grid, 256, 0, st>>>(src, ldca, words, d.k_log2, fresh);
+  else if (src.count == 1 && src.s[0].planes && !src.s[0].ldca)
+    k_fold8<false><<<2 * grid, kFold8Threads, 0, st>>>(src, ldca, words, d.k_log2, fresh);
+  else k_fold8<true><<<2 * grid, kFold8Threads, 0, st>>>(src, ldca, words, d.k_log2, fresh);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_fold(const DevParams& d, const uint32_t* planes, uint32_t* ldca, int grid, cudaStream_t st,
                         const uint32_t* fresh) {
-  const uint32_t words = (uint32_t)(((uint64_t)d.lr << d.lc_log2) >> 5);
-  if (d.k_log2 >= 8) k_fold8<<<grid, 256, 0, st>>>(planes, ldca, words, d.k_log2, fresh);
-  else k_fold<<<grid, 256, 0, st>>>(planes, ldca, words, d.k_log2, fresh);
-  return cudaGetLastError();
+  FoldSrcs src{};
+  src.s[0].planes = planes;
+  src.count = 1;
+  return launch_fold_multi(d, src, ldca, grid, st, fresh);
 }
 
 BinSrc bin_src_one(const uint32_t* pairs, uint64_t n_pairs) {
