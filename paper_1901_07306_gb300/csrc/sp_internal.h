@@ -58,11 +58,12 @@ __host__ __device__ __forceinline__ uint32_t gather_idx(uint32_t lp, uint32_t is
 }
 
 // Up to kBinMaxSrc streams of one router, binned by one k_bin launch.
-constexpr int kBinMaxSrc = 32;
+constexpr int kBinMaxSrc = 128;       // a multiple of 32
 struct BinSrc {
   const uint32_t* ptr[kBinMaxSrc];
   uint64_t n[kBinMaxSrc];
   uint32_t count;
+  uint32_t full_max, small_quads;   // whole tiles taken of a stream, quads of a small tile (binned_bin_chunk)
 };
 
 // Staging shape of the binned scan (sp_scan_binned.cu); every compiled shape
@@ -118,9 +119,10 @@ uint32_t binned_list_cap(uint64_t n_pairs, uint32_t bins, const BinShape& shape,
 uint32_t binned_tile_pairs(const BinShape& shape);
 // bytes of one router's plane accumulator ([ceil(W / 8)][k][8] words)
 uint64_t binned_planes_bytes(const DevParams& d);
-// one binning launch over pairs[0, n) into the lists (append: continue them)
-cudaError_t binned_bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, const BinSrc& src,
-                             const BinnedScratch& s, uint32_t cap, bool append, uint32_t rot, cudaStream_t st);
+// one binning launch over the streams into the lists (append: continue them);
+// *rot: tiles of the round's earlier launches, so that blocks take turns
+cudaError_t binned_bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, BinSrc& src,
+                             const BinnedScratch& s, uint32_t cap, bool append, uint64_t* rot, cudaStream_t st);
 BinSrc bin_src_one(const uint32_t* pairs, uint64_t n_pairs);
 // the planes of the lists' hips (accumulate: on top of the pending planes)
 cudaError_t binned_apply_round(const DevParams& d, const BinnedScratch& s, uint32_t cap, bool accumulate,

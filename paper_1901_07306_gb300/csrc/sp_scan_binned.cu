@@ -45,7 +45,6 @@ namespace {
 constexpr int kVec = 4;                            // 16-byte loads (2 pairs) per thread and tile
 constexpr int kGroup = 4;                          // pairs hashed and staged together
 constexpr int kChunk = 8;                          // hips per list store (32 bytes)
-constexpr int kApplyUnroll = 8;                    // hip loads in flight per lane
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 
 __device__ __forceinline__ void seav_set(const DevParams& d, uint8_t* seav, uint32_t hip, uint32_t h1) {
@@ -83,8 +82,8 @@ __device__ __forceinline__ void st_chunk(uint32_t* dst, uint4 a, uint4 b) {
 // k_bin: tiles of TILE = THREADS * 2 kVec pairs, tile (slot + i G) in iteration i.  Each
 // thread holds kVec 16-byte loads (2 pairs each) of a tile in registers and
 // issues the loads of tile i + 1 before it works on tile i, so the copy from
-// HBM overlaps the work.  Tiles that are partial, or a stream that is not
-// 16-byte aligned, are read pair by pair instead.  Every bin owns a staging
+// HBM overlaps the work.  What is left after whole rounds over the blocks is
+// cut into one small tile for each block.  Every bin owns a staging
 // row of STAGE hips in shared memory that persists across tiles (a
 // write-combining buffer for the bin's list).  Per tile:
 //   1. every thread hashes its pairs, queues the sampled pairs (Sec. 3.1) for
@@ -103,7 +102,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
 k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
       BinSrc src, uint32_t* __restrict__ lists, uint32_t* __restrict__ counts, uint32_t cap,
       bool append, uint32_t rot, uint32_t* __restrict__ ovf) {
-  constexpr int TILE = THREADS * kVec * 2;
+  constexpr int QUADS = THREADS * kVec;               // 16-byte loads of a whole tile
+  constexpr int TILE = QUADS * 2;
   constexpr int QUEUE = TPR * TILE / 32;              // sampled pairs per round: 4x the expected 2^-7
   extern __shared__ __align__(128) uint8_t smem_raw[];
   const uint32_t bins = 1u << d.k_log2;                                // <= 1024
@@ -113,7 +113,7 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
   uint32_t* s_fill = reinterpret_cast<uint32_t*>(s_queue + QUEUE);     // [bins] hips in the row
   uint32_t* s_cursor = s_fill + bins;                                   // [bins] list fill (whole chunks)
   __shared__ uint32_t s_qn[2];                                          // queue fill, by tile parity
-  __shared__ uint64_t s_tpref[kBinMaxSrc + 1];
+  __shared__ uint32_t s_full[kBinMaxSrc + 1], s_small[kBinMaxSrc + 1];   // tiles before stream b (fewer than 2^32 a round)
   const uint32_t tid = threadIdx.x;
   const uint32_t G = gridDim.x, cta = blockIdx.x;
   const uint32_t slot = (cta + rot) % G;          // which tiles this block takes
@@ -128,15 +128,37 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
     ldca_red(d, ldca, hip, b);
     if (ovf) *ovf = 1u;
   };
-  // tiles of the streams, back to back: stream b owns tiles [s_tpref[b], s_tpref[b + 1])
-  if (tid == 0) {
-    uint64_t acc = 0;
-    s_tpref[0] = 0;
-    for (uint32_t b = 0; b < src.count; ++b) {
-      acc += (src.n[b] + TILE - 1) / TILE;
-      s_tpref[b + 1] = acc;
+  // A stream is a body of 16-byte quads (two pairs) and up to two single
+  // pairs: its first one when it starts 8 bytes off a 16-byte boundary, its last
+  // one when one is left over.  The body is cut into whole tiles (at most
+  // src.full_max of a stream) and small ones of src.small_quads for the rest;
+  // whole tiles of stream b are [s_full[b], s_full[b + 1]), small ones likewise.
+  auto head_of = [&](uint32_t b) { return ((uintptr_t)src.ptr[b] & 15u) != 0u ? 1u : 0u; };
+  auto quads_of = [&](uint32_t b) { return src.n[b] != 0 ? (src.n[b] - head_of(b)) >> 1 : (uint64_t)0; };
+  if (tid < 64) {                                  // warp 0: whole tiles, warp 1: small ones
+    uint32_t* pref = tid < 32 ? s_full : s_small;
+    uint32_t sum[kBinMaxSrc / 32], acc = 0;
+#pragma unroll
+    for (int e = 0; e < kBinMaxSrc / 32; ++e) {
+      const uint32_t b = lane * (kBinMaxSrc / 32) + (uint32_t)e;
+      if (b < src.count) {
+        const uint64_t quads = quads_of(b);
+        const uint32_t full = (uint32_t)min(quads / QUADS, (uint64_t)src.full_max);
+        acc += tid < 32 ? full
+                        : (uint32_t)((quads - (uint64_t)full * QUADS + src.small_quads - 1) / src.small_quads);
+      }
+      sum[e] = acc;
     }
-    s_qn[0] = s_qn[1] = 0;
+    uint32_t incl = acc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= (uint32_t)o) incl += y;
+    }
+#pragma unroll
+    for (int e = 0; e < kBinMaxSrc / 32; ++e) pref[lane * (kBinMaxSrc / 32) + (uint32_t)e + 1] = incl - acc + sum[e];
+    if (lane == 0) pref[0] = 0;
+    if (tid == 0) s_qn[0] = s_qn[1] = 0;
   }
   auto list_of = [&](uint32_t b) { return lists + ((uint64_t)b * G + cta) * cap; };
   for (uint32_t b = tid; b < bins; b += THREADS) {
@@ -148,27 +170,16 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
     s_cursor[b] = have - tail;
   }
   __syncthreads();
-  const uint64_t n_tiles = s_tpref[src.count];
-  auto tile_of = [&](uint64_t i) { return (uint64_t)slot + i * G; };
-  // a tile: its first pair, its pair count, whether it is read with 16-byte loads
-  struct TileRef { const uint2* p; uint32_t n; bool vec; };
-  uint32_t stream_hint = 0;                      // this block's tiles come in stream order
-  auto tile_ref = [&](uint64_t tile) {
-    uint32_t b = stream_hint;
-    while (s_tpref[b + 1] <= tile) ++b;
-    stream_hint = b;
-    const uint64_t base = (tile - s_tpref[b]) * TILE;
-    const uint64_t left = src.n[b] - base;
-    TileRef t;
-    t.p = reinterpret_cast<const uint2*>(src.ptr[b]) + base;
-    t.n = left < (uint64_t)TILE ? (uint32_t)left : (uint32_t)TILE;
-    t.vec = ((uintptr_t)src.ptr[b] & 15u) == 0 && t.n == (uint32_t)TILE;
-    return t;
-  };
+  const uint32_t n_tiles = s_full[src.count], n_small = s_small[src.count];
   // 16-byte streaming loads of this thread's share of a whole tile; volatile,
   // so they are issued where they stand (before the work on the previous tile)
-  auto load_tile = [&](uint4 (&r)[kVec], const uint2* p) {
-    const uint4* p4 = reinterpret_cast<const uint4*>(p) + tid;
+  uint32_t stream_hint = 0;                      // this block's tiles come in stream order
+  auto load_tile = [&](uint4 (&r)[kVec], uint32_t tile) {
+    uint32_t b = stream_hint;
+    while (s_full[b + 1] <= tile) ++b;
+    stream_hint = b;
+    const uint4* p4 = reinterpret_cast<const uint4*>(src.ptr[b] + 2u * head_of(b)) +
+                      (uint64_t)(tile - s_full[b]) * QUADS + tid;
 #pragma unroll
     for (int u = 0; u < kVec; ++u)
       asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];"
@@ -242,34 +253,19 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
     s_fill[b] = rem;
     s_cursor[b] = cur;
   };
-  // 1. hash, queue the sampled pairs, stage the hips of one tile in their bins' rows
-  auto stage_tile = [&](const uint4 (&r)[kVec], const TileRef& t, uint32_t par) {
-    if (t.vec) {
+  // 1. hash, queue the sampled pairs, stage the hips of one whole tile in their bins' rows
+  auto stage_tile = [&](const uint4 (&r)[kVec], uint32_t par) {
 #pragma unroll
-      for (int g = 0; g < kVec / (kGroup / 2); ++g) {
-        uint32_t hip[kGroup], oip[kGroup], bin[kGroup];
+    for (int g = 0; g < kVec / (kGroup / 2); ++g) {
+      uint32_t hip[kGroup], oip[kGroup], bin[kGroup];
 #pragma unroll
-        for (int u = 0; u < kGroup / 2; ++u) {
-          const uint4 v = r[g * (kGroup / 2) + u];
-          hip[2 * u] = v.x; oip[2 * u] = v.y;
-          hip[2 * u + 1] = v.z; oip[2 * u + 1] = v.w;
-        }
-        const uint32_t over = stage_group(hip, oip, (1u << kGroup) - 1u, par, bin);
-        group_leftovers(hip, oip, bin, over);
+      for (int u = 0; u < kGroup / 2; ++u) {
+        const uint4 v = r[g * (kGroup / 2) + u];
+        hip[2 * u] = v.x; oip[2 * u] = v.y;
+        hip[2 * u + 1] = v.z; oip[2 * u + 1] = v.w;
       }
-    } else {
-      for (uint32_t j0 = 0; j0 < (uint32_t)TILE; j0 += kGroup * THREADS) {
-        uint32_t hip[kGroup], oip[kGroup], bin[kGroup], valid = 0;
-#pragma unroll
-        for (int q = 0; q < kGroup; ++q) {
-          const uint32_t j = j0 + (uint32_t)q * THREADS + tid;
-          uint2 v = make_uint2(0u, 0u);
-          if (j < t.n) { v = __ldcs(t.p + j); valid |= 1u << q; }
-          hip[q] = v.x; oip[q] = v.y;
-        }
-        const uint32_t over = stage_group(hip, oip, valid, par, bin);
-        group_leftovers(hip, oip, bin, over);
-      }
+      const uint32_t over = stage_group(hip, oip, (1u << kGroup) - 1u, par, bin);
+      group_leftovers(hip, oip, bin, over);
     }
   };
   // the flush round: whole chunks to the lists; the queued SEAV updates,
@@ -292,57 +288,95 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
   // for tile t + 2 go out as soon as tile t is staged, so the flush round
   // runs with both next tiles in flight (the flush's stores and the stream's
   // loads overlap); a flush round after every TPR tiles.
-  uint4 ra[kVec], rb[kVec];
-  TileRef ta{nullptr, 0u, false}, tb{nullptr, 0u, false};
-  if (tile_of(0) < n_tiles) {
-    ta = tile_ref(tile_of(0));
-    if (ta.vec) load_tile(ra, ta.p);
-  }
-  if (tile_of(1) < n_tiles) {
-    tb = tile_ref(tile_of(1));
-    if (tb.vec) load_tile(rb, tb.p);
-  }
   uint32_t par = 0;
-  for (uint64_t i = 0; tile_of(i) < n_tiles; i += 2) {
-    const bool has_b = tile_of(i + 1) < n_tiles;
-    stage_tile(ra, ta, par);
-    if (tile_of(i + 2) < n_tiles) {
-      ta = tile_ref(tile_of(i + 2));
-      if (ta.vec) load_tile(ra, ta.p);
-    }
-    if (TPR == 1) {
+  if (slot < n_tiles) {
+    uint4 ra[kVec], rb[kVec];
+    load_tile(ra, slot);
+    if (slot + G < n_tiles) load_tile(rb, slot + G);
+    for (uint32_t t = slot; t < n_tiles; t += 2 * G) {
+      stage_tile(ra, par);
+      if (t + 2 * G < n_tiles) load_tile(ra, t + 2 * G);
+      if (TPR == 1) {
+        flush_round(par);
+        par ^= 1u;
+      }
+      if (t + G < n_tiles) {
+        stage_tile(rb, par);
+        if (t + 3 * G < n_tiles) load_tile(rb, t + 3 * G);
+      }
       flush_round(par);
       par ^= 1u;
     }
-    if (has_b) {
-      stage_tile(rb, tb, par);
-      if (tile_of(i + 3) < n_tiles) {
-        tb = tile_ref(tile_of(i + 3));
-        if (tb.vec) load_tile(rb, tb.p);
+  }
+  // small tiles, first to the blocks that had a whole tile less, and the
+  // streams' single pairs with them: all of a thread's loads, then the work
+  for (uint32_t t = (slot + G - n_tiles % G) % G; t < n_small || t < src.count; t += G) {
+    uint32_t b = 0, n = 0;
+    uint4 r[kVec];
+    if (t < n_small) {
+      while (s_small[b + 1] <= t) ++b;
+      const uint64_t base = (uint64_t)(s_full[b + 1] - s_full[b]) * QUADS + (uint64_t)(t - s_small[b]) * src.small_quads;
+      n = (uint32_t)min(quads_of(b) - base, (uint64_t)src.small_quads);
+      const uint4* p4 = reinterpret_cast<const uint4*>(src.ptr[b] + 2u * head_of(b)) + base;
+#pragma unroll
+      for (int u = 0; u < kVec; ++u)
+        if (tid + u * THREADS < n) r[u] = __ldcs(p4 + tid + u * THREADS);
+    }
+#pragma unroll
+    for (int g = 0; g <= kVec / (kGroup / 2); ++g) {
+      uint32_t hip[kGroup] = {}, oip[kGroup] = {}, bin[kGroup], valid = 0;
+      if (g < kVec / (kGroup / 2)) {
+#pragma unroll
+        for (int u = 0; u < kGroup / 2; ++u) {
+          const int q = g * (kGroup / 2) + u;
+          if (tid + (uint32_t)q * THREADS < n) {
+            hip[2 * u] = r[q].x; oip[2 * u] = r[q].y;
+            hip[2 * u + 1] = r[q].z; oip[2 * u + 1] = r[q].w;
+            valid |= 3u << (2 * u);
+          }
+        }
+      } else if (t < src.count && tid < 2) {          // stream t: thread 0 its first pair, thread 1 its last one
+        const uint32_t head = head_of(t);
+        if (src.n[t] != 0 && (tid == 0 ? head != 0u : ((src.n[t] - head) & 1u) != 0u)) {
+          const uint2 v = reinterpret_cast<const uint2*>(src.ptr[t])[tid == 0 ? 0 : src.n[t] - 1];
+          hip[0] = v.x; oip[0] = v.y;
+          valid = 1u;
+        }
+      }
+      if (__any_sync(kFull, valid != 0u)) {
+        const uint32_t over = stage_group(hip, oip, valid, par, bin);
+        group_leftovers(hip, oip, bin, over);
       }
     }
     flush_round(par);
     par ^= 1u;
   }
-  // remainders (< 8 hips per row) with plain stores
+  // remainders (< 8 hips per row): one more chunk, filled up with copies of a
+  // hip of its own, so that k_apply reads whole 16-byte quads of a list (a bit
+  // set twice is the same bit); counts[] has the real number
   for (uint32_t b = tid; b < bins; b += THREADS) {
-    const uint32_t f = s_fill[b];
-    uint32_t* list = list_of(b);
-    uint32_t c = s_cursor[b];
-    for (uint32_t e = 0; e < f; ++e) {
-      const uint32_t h = stage[b * STAGE + e];
-      if (c < cap) list[c++] = h;
-      else spill(h, b);
+    const uint32_t f = s_fill[b], c = s_cursor[b];
+    const uint32_t* row = stage + b * STAGE;
+    uint32_t kept = 0;
+    if (f != 0u && c + kChunk <= cap) {
+      const uint4 x = *reinterpret_cast<const uint4*>(row), y = *reinterpret_cast<const uint4*>(row + 4);
+      st_chunk(list_of(b) + c,
+               make_uint4(x.x, f > 1 ? x.y : x.x, f > 2 ? x.z : x.x, f > 3 ? x.w : x.x),
+               make_uint4(f > 4 ? y.x : x.x, f > 5 ? y.y : x.x, f > 6 ? y.z : x.x, x.x));
+      kept = f;
+    } else {
+      for (uint32_t e = 0; e < f; ++e) spill(row[e], b);
     }
-    counts[(uint64_t)b * G + cta] = c;
+    counts[(uint64_t)b * G + cta] = c + kept;
   }
 }
 
 // A list read once streams past L2 (evict first); a list that SPLIT > 1
 // blocks read, close together in time, stays there for the second read.
 template <int SPLIT>
-__device__ __forceinline__ uint32_t load_hip(const uint32_t* p) {
-  return SPLIT == 1 ? __ldcs(p) : __ldg(p);
+__device__ __forceinline__ uint4 load_hips(const uint32_t* p) {
+  const uint4* q = reinterpret_cast<const uint4*>(p);
+  return SPLIT == 1 ? __ldcs(q) : __ldg(q);
 }
 
 // k_apply, LCL = log2 LC when it is fixed at compile time (profiles D, D3
@@ -350,31 +384,37 @@ __device__ __forceinline__ uint32_t load_hip(const uint32_t* p) {
 // a plane, each holding LR / SPLIT of its LDCA rows in shared memory and
 // reading the whole hip list: wide planes (LC = 2^18: 128 KiB for four rows)
 // would otherwise leave one block per SM.
+// Groups of 8 lanes walk the plane's lists on their own, 32 hips a step, one
+// 16-byte load per lane, issued a step ahead, so that short lists -- a launch
+// of 5 M pairs leaves 32 hips in each -- cost one load's latency for the whole
+// plane and not one count and one load per list and warp; the lists' counts
+// are in shared memory before the walk starts.  A group takes whole lists:
+// sharing one among 2 or 4 groups balances the warps better and measured 3%
+// slower (more ragged ends), two loads per lane and step the same.
+// Lists are filled up to whole 8-hip chunks (k_bin), so a lane's 4 hips are
+// all there or none is.
 template <int LR, int THREADS, int LCL, int SPLIT>
 __global__ void __launch_bounds__(THREADS)
 k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restrict__ counts,
         uint32_t G, uint32_t cap, uint32_t* __restrict__ planes, bool accumulate) {
-  extern __shared__ uint32_t s_plane[];
+  extern __shared__ __align__(16) uint32_t s_plane[];
   constexpr int LRP = LR / SPLIT;                                  // rows of this block
+  constexpr uint32_t NG = THREADS / 8;
   const uint32_t b = blockIdx.x / SPLIT;
   const uint32_t row0 = (blockIdx.x % SPLIT) * (uint32_t)LRP;
   const uint32_t lc_log2 = LCL ? (uint32_t)LCL : d.lc_log2;
-  const uint32_t words = ((uint32_t)LRP << lc_log2) >> 5;         // words of the block's rows
-  const uint32_t word0 = row0 << (lc_log2 - 5u);                  // their first plane word
-  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-  const uint32_t nwarps = THREADS / 32;
+  const uint32_t chunks = ((((uint32_t)LRP << lc_log2) >> 5) + 7u) / 8u;  // 8-word chunks of the block's rows
+  uint32_t* s_count = s_plane + chunks * 8u;                       // [G]
+  const uint32_t tid = threadIdx.x, lane = tid & 31u;
   // LH_i(hip) = h >> cshift (5 <= lc_log2 <= 20): LDC h >> cshift of row i is
   // bit (h >> cshift) mod 32 of plane word (i << (lc_log2 - 5)) + (h >> (cshift + 5))
   const uint32_t cshift = 32u - lc_log2;
   const uint32_t row_words_log2 = lc_log2 - 5u;
   // accumulator layout [ceil(words / 8)][k][8]: word w of plane b at
-  // (w / 8) k 8 + 8 b + w mod 8, so that a 32-byte chunk holds 8 words of one plane
+  // (w / 8) k 8 + 8 b + w mod 8, so that a 32-byte chunk holds 8 words of one
+  // plane (with SPLIT > 1 a row is a multiple of 8 words)
   const uint64_t chunk_stride = (uint64_t)(1u << d.k_log2) * 8u;
-  uint32_t* dst = planes + (uint64_t)b * 8u;
-  auto at_word = [&](uint32_t w) {
-    w += word0;
-    return dst + (uint64_t)(w >> 3) * chunk_stride + (w & 7u);
-  };
+  uint32_t* dst = planes + (uint64_t)b * 8u + (uint64_t)((row0 << row_words_log2) / 8u) * chunk_stride;
   // the rows' hash words, held in registers
   uint32_t a_lo[LRP], a_hi[LRP];
   uint64_t bw[LRP];
@@ -384,7 +424,17 @@ k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restr
     a_hi[r] = (uint32_t)(d.ha[2 + row0 + r] >> 32);
     bw[r] = d.hb[2 + row0 + r];
   }
-  for (uint32_t w = tid; w < words; w += THREADS) s_plane[w] = accumulate ? *at_word(w) : 0u;
+  for (uint32_t c = tid; c < G; c += THREADS) s_count[c] = counts[(uint64_t)b * G + c];
+  for (uint32_t ch = tid; ch < chunks; ch += THREADS) {
+    uint4 x = make_uint4(0u, 0u, 0u, 0u), y = x;
+    if (accumulate) {
+      const uint4* p = reinterpret_cast<const uint4*>(dst + ch * chunk_stride);
+      x = p[0];
+      y = p[1];
+    }
+    *reinterpret_cast<uint4*>(s_plane + ch * 8u) = x;
+    *reinterpret_cast<uint4*>(s_plane + ch * 8u + 4u) = y;
+  }
   __syncthreads();
   auto set_bits = [&](uint32_t hip) {
 #pragma unroll
@@ -401,29 +451,39 @@ k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restr
       }
     }
   };
-  for (uint32_t c = warp; c < G; c += nwarps) {
-    const uint32_t n = counts[(uint64_t)b * G + c];
-    const uint32_t* src = lists + ((uint64_t)b * G + c) * cap + lane;
-    uint32_t i0 = 0;
-    for (; i0 + 32 * kApplyUnroll <= n; i0 += 32 * kApplyUnroll) {     // whole rounds: no bounds checks
-      uint32_t hip[kApplyUnroll];
-#pragma unroll
-      for (int u = 0; u < kApplyUnroll; ++u) hip[u] = load_hip<SPLIT>(src + i0 + u * 32);   // all in flight
-#pragma unroll
-      for (int u = 0; u < kApplyUnroll; ++u) set_bits(hip[u]);
+  const uint32_t first = 4u * (lane & 7u);                          // this lane's hips of a step: first .. first + 3
+  uint32_t c = tid >> 3, at = first;
+  uint32_t n = c < G ? s_count[c] : 0u;
+  const uint32_t* list = lists + ((uint64_t)b * G + c) * cap;
+  uint4 cur = make_uint4(0u, 0u, 0u, 0u);
+  bool have = at < n;
+  if (have) cur = load_hips<SPLIT>(list + at);
+  bool live = c < G;
+  while (__any_sync(kFull, live)) {
+    at += 32u;
+    if (at - first >= n) {                                          // the group's next list
+      c += NG;
+      at = first;
+      n = c < G ? s_count[c] : 0u;
+      list += (uint64_t)NG * cap;
     }
-    if (i0 < n) {                                   // the last, partial round: masked, loads still in flight together
-      uint32_t hip[kApplyUnroll];
-#pragma unroll
-      for (int u = 0; u < kApplyUnroll; ++u)
-        hip[u] = (i0 + u * 32 + lane < n) ? load_hip<SPLIT>(src + i0 + u * 32) : 0u;
-#pragma unroll
-      for (int u = 0; u < kApplyUnroll; ++u)
-        if (i0 + u * 32 + lane < n) set_bits(hip[u]);
+    live = c < G;
+    const bool more = at < n;
+    uint4 next = cur;
+    if (more) next = load_hips<SPLIT>(list + at);
+    if (have) {
+      set_bits(cur.x);
+      set_bits(cur.y);
+      set_bits(cur.z);
+      set_bits(cur.w);
     }
+    cur = next;
+    have = more;
   }
   __syncthreads();
-  for (uint32_t w = tid; w < words; w += THREADS) *at_word(w) = s_plane[w];
+  for (uint32_t ch = tid; ch < chunks; ch += THREADS)
+    st_chunk(dst + ch * chunk_stride, *reinterpret_cast<const uint4*>(s_plane + ch * 8u),
+             *reinterpret_cast<const uint4*>(s_plane + ch * 8u + 4u));
 }
 
 // 32 x 32 bit transpose across a warp: lane l holds row l (bit j = column j);
@@ -659,8 +719,8 @@ cudaError_t bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, const B
 template <int LR, int THREADS, int LCL, int SPLIT = 1>
 cudaError_t apply_round_t(const DevParams& d, const BinnedScratch& s, uint32_t cap, bool accumulate, cudaStream_t st) {
   const uint32_t bins = 1u << d.k_log2;
-  const uint32_t words = ((uint32_t)(LR / SPLIT) << d.lc_log2) >> 5;
-  const size_t apply_smem = (size_t)words * sizeof(uint32_t);
+  const uint32_t chunks = ((((uint32_t)(LR / SPLIT) << d.lc_log2) >> 5) + 7u) / 8u;
+  const size_t apply_smem = ((size_t)chunks * 8u + s.ctas) * sizeof(uint32_t);   // the rows, the lists' counts
   auto kern = k_apply<LR, THREADS, LCL, SPLIT>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem);
   if (e != cudaSuccess) return e;
@@ -757,15 +817,31 @@ BinSrc bin_src_one(const uint32_t* pairs, uint64_t n_pairs) {
   return src;
 }
 
-cudaError_t binned_bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, const BinSrc& src,
-                             const BinnedScratch& s, uint32_t cap, bool append, uint32_t rot, cudaStream_t st) {
+cudaError_t binned_bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, BinSrc& src,
+                             const BinnedScratch& s, uint32_t cap, bool append, uint64_t* rot, cudaStream_t st) {
   if (src.count == 0) return cudaSuccess;
   // the list stride never exceeds what was allocated (hips past a full list go
   // to L2 REDs, so a smaller cap only costs speed)
   if (cap > s.cap_alloc) cap = s.cap_alloc;
   const BinShape& h = s.shape;
-  if (h.threads == 512) return bin_chunk<512, 20, 2, 2>(d, seav, ldca, src, s, cap, append, rot, st);
-  return bin_chunk<1024, 44, 2, 1>(d, seav, ldca, src, s, cap, append, rot, st);
+  // Whole tiles as long as they make whole rounds over the blocks; the rest in
+  // small tiles, one for each block (whole warps of quads).  Streams of a
+  // batched launch keep all their whole tiles.
+  const uint64_t most = binned_tile_pairs(h) / 2;
+  uint64_t quads = 0, full = 0;
+  for (uint32_t b = 0; b < src.count; ++b) {
+    quads += src.n[b] / 2;
+    full += src.n[b] / 2 / most;
+  }
+  if (src.count == 1) full = full / s.ctas * s.ctas;
+  src.full_max = src.count == 1 ? (uint32_t)full : 0xFFFFFFFFu;
+  uint64_t small = (quads - full * most + s.ctas - 1) / s.ctas;
+  small = (small + 31) & ~31ull;
+  src.small_quads = (uint32_t)(small < 32 ? 32 : small > most ? most : small);
+  const uint32_t r = (uint32_t)(*rot % s.ctas);
+  *rot += full + s.ctas - 1;
+  if (h.threads == 512) return bin_chunk<512, 20, 2, 2>(d, seav, ldca, src, s, cap, append, r, st);
+  return bin_chunk<1024, 44, 2, 1>(d, seav, ldca, src, s, cap, append, r, st);
 }
 
 cudaError_t binned_apply_round(const DevParams& d, const BinnedScratch& s, uint32_t cap, bool accumulate,
@@ -797,7 +873,9 @@ cudaError_t launch_scan_binned(const DevParams& d, uint8_t* seav, uint32_t* ldca
   while (done < n_pairs) {
     const uint64_t n = (n_pairs - done) < s.max_pairs ? (n_pairs - done) : s.max_pairs;
     const uint32_t cap = binned_list_cap(n, 1u << d.k_log2, s.shape, s.ctas, 1);
-    cudaError_t e = binned_bin_chunk(d, seav, ldca, bin_src_one(pairs + 2 * done, n), s, cap, false, 0, st);
+    BinSrc src = bin_src_one(pairs + 2 * done, n);
+    uint64_t rot = 0;
+    cudaError_t e = binned_bin_chunk(d, seav, ldca, src, s, cap, false, &rot, st);
     if (e == cudaSuccess) e = binned_apply_round(d, s, cap, accumulate, st);
     if (e != cudaSuccess) return e;
     accumulate = true;
