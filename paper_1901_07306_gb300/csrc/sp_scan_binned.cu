@@ -34,7 +34,10 @@
 // tiles, or two 512-thread blocks per SM with 20-hip rows flushing every tile,
 // so one block's flush overlaps the other's hashing -- and the k_apply block
 // size.
+#include <cuda.h>
 #include <math.h>
+
+#include <atomic>
 
 #include "sp_internal.h"
 
@@ -396,8 +399,9 @@ __device__ __forceinline__ uint4 load_hips(const uint32_t* p) {
 template <int LR, int THREADS, int LCL, int SPLIT>
 __global__ void __launch_bounds__(THREADS)
 k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restrict__ counts,
-        uint32_t G, uint32_t cap, uint32_t* __restrict__ planes, bool accumulate) {
-  extern __shared__ __align__(16) uint32_t s_plane[];
+        uint32_t G, uint32_t cap, const uint32_t* planes, const __grid_constant__ CUtensorMap map, uint32_t box,
+        bool accumulate) {
+  extern __shared__ __align__(128) uint32_t s_plane[];
   constexpr int LRP = LR / SPLIT;                                  // rows of this block
   constexpr uint32_t NG = THREADS / 8;
   const uint32_t b = blockIdx.x / SPLIT;
@@ -414,7 +418,8 @@ k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restr
   // (w / 8) k 8 + 8 b + w mod 8, so that a 32-byte chunk holds 8 words of one
   // plane (with SPLIT > 1 a row is a multiple of 8 words)
   const uint64_t chunk_stride = (uint64_t)(1u << d.k_log2) * 8u;
-  uint32_t* dst = planes + (uint64_t)b * 8u + (uint64_t)((row0 << row_words_log2) / 8u) * chunk_stride;
+  const uint32_t chunk0 = (row0 << row_words_log2) / 8u;            // the block's first chunk
+  const uint32_t* src = planes + (uint64_t)b * 8u + (uint64_t)chunk0 * chunk_stride;
   // the rows' hash words, held in registers
   uint32_t a_lo[LRP], a_hi[LRP];
   uint64_t bw[LRP];
@@ -425,16 +430,10 @@ k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restr
     bw[r] = d.hb[2 + row0 + r];
   }
   for (uint32_t c = tid; c < G; c += THREADS) s_count[c] = counts[(uint64_t)b * G + c];
-  for (uint32_t ch = tid; ch < chunks; ch += THREADS) {
-    uint4 x = make_uint4(0u, 0u, 0u, 0u), y = x;
-    if (accumulate) {
-      const uint4* p = reinterpret_cast<const uint4*>(dst + ch * chunk_stride);
-      x = p[0];
-      y = p[1];
-    }
-    *reinterpret_cast<uint4*>(s_plane + ch * 8u) = x;
-    *reinterpret_cast<uint4*>(s_plane + ch * 8u + 4u) = y;
-  }
+  for (uint32_t u = tid; u < chunks * 2u; u += THREADS)             // 16-byte units, consecutive lanes
+    *reinterpret_cast<uint4*>(s_plane + u * 4u) =
+        accumulate ? *reinterpret_cast<const uint4*>(src + (u >> 1) * chunk_stride + (u & 1u) * 4u)
+                   : make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
   auto set_bits = [&](uint32_t hip) {
 #pragma unroll
@@ -480,10 +479,19 @@ k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restr
     cur = next;
     have = more;
   }
+  // the plane's chunks go out by TMA, `box` chunks a copy: 1,024 sectors 32 KiB
+  // apart (profile D), which as 32-byte stores took one wavefront of the
+  // load-store pipe each, the pipe that bounds the kernel
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
-  for (uint32_t ch = tid; ch < chunks; ch += THREADS)
-    st_chunk(dst + ch * chunk_stride, *reinterpret_cast<const uint4*>(s_plane + ch * 8u),
-             *reinterpret_cast<const uint4*>(s_plane + ch * 8u + 4u));
+  if (tid == 0) {
+    for (uint32_t ch = 0; ch < chunks; ch += box)
+      asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+                   :: "l"(&map), "r"(0), "r"(b), "r"(chunk0 + ch),
+                      "r"((uint32_t)__cvta_generic_to_shared(s_plane + ch * 8u)) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // shared memory is read before the block ends
+  }
 }
 
 // 32 x 32 bit transpose across a warp: lane l holds row l (bit j = column j);
@@ -716,6 +724,30 @@ cudaError_t bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, const B
   return cudaGetLastError();
 }
 
+// The accumulator as a tensor [chunks][bins][8] of words; copies take `box`
+// chunks of one plane.
+cudaError_t plane_map(uint32_t* planes, uint32_t bins, uint32_t chunks, uint32_t box, CUtensorMap* map) {
+  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static std::atomic<void*> entry{nullptr};
+  void* fn = entry.load(std::memory_order_acquire);
+  if (fn == nullptr) {
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    const cudaError_t e =
+        cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
+    if (e != cudaSuccess) return e;
+    if (found != cudaDriverEntryPointSuccess || fn == nullptr) return cudaErrorSymbolNotFound;
+    entry.store(fn, std::memory_order_release);
+  }
+  const cuuint64_t dims[3] = {8, bins, chunks}, strides[2] = {32, (cuuint64_t)bins * 32};
+  const cuuint32_t boxes[3] = {8, 1, box}, steps[3] = {1, 1, 1};
+  const CUresult r = reinterpret_cast<Encode>(fn)(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, planes, dims, strides, boxes,
+                                                  steps, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 template <int LR, int THREADS, int LCL, int SPLIT = 1>
 cudaError_t apply_round_t(const DevParams& d, const BinnedScratch& s, uint32_t cap, bool accumulate, cudaStream_t st) {
   const uint32_t bins = 1u << d.k_log2;
@@ -724,7 +756,12 @@ cudaError_t apply_round_t(const DevParams& d, const BinnedScratch& s, uint32_t c
   auto kern = k_apply<LR, THREADS, LCL, SPLIT>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem);
   if (e != cudaSuccess) return e;
-  kern<<<bins * SPLIT, THREADS, apply_smem, st>>>(d, s.lists, s.counts, s.ctas, cap, s.planes, accumulate);
+  // chunks of a copy: a block's chunks in equal boxes of at most 256
+  uint32_t box = chunks < 256u ? chunks : 256u;
+  while (chunks % box != 0u) --box;
+  CUtensorMap map;
+  if ((e = plane_map(s.planes, bins, chunks * (uint32_t)SPLIT, box, &map)) != cudaSuccess) return e;
+  kern<<<bins * SPLIT, THREADS, apply_smem, st>>>(d, s.lists, s.counts, s.ctas, cap, s.planes, map, box, accumulate);
   return cudaGetLastError();
 }
 
