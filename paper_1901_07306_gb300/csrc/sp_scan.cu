@@ -71,6 +71,112 @@ k_scan(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
   }
 }
 
+// ---- the direct form with the heavy hosts held on chip ----------------------
+//
+// A host's pairs all hit its LR LDC lines, and the REDs of one line are
+// serialised in its L2 slice at about 1.25 ns apiece: one host with 50,000 of
+// 2^20 pairs took 63 us, against 20 us for the window's 2^22 REDs at the rate
+// of random lines.  Every pair of a host sets the same bit H3(oip) in each of
+// its lines, so a block keeps one vector of k bits per heavy host in shared
+// memory (one shared atomic per pair) and ORs its nonzero words into the LR
+// lines once, at the end.  Heavy are the hosts that appear at least `heavy`
+// times among the block's first 2,048 pairs (one pass through a direct-mapped
+// table, which afterwards answers the lookups); all others go to REDs as
+// before, so any input gives the same bits.
+constexpr int kHotThreads = 1024;
+constexpr uint32_t kHotSlots = 2048;               // the table (16 KiB)
+constexpr uint32_t kHotWords = 4096;               // the vectors (16 KiB)
+constexpr uint32_t kHotMax = 64;                   // hosts held, k permitting
+constexpr uint32_t kNoHost = 0xFFFFFFFFu;          // marks a free slot; that address itself is never held
+constexpr uint64_t kHotPairs = 1ull << 18;         // updates from here on (scan_launch)
+
+template <int LR>
+__global__ void __launch_bounds__(kHotThreads)
+k_scan_hot(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
+           const uint32_t* __restrict__ pairs, uint64_t n_pairs, uint32_t heavy) {
+  __shared__ uint2 s_tab[kHotSlots];               // (host, 1 + index of its vector or 0)
+  __shared__ uint32_t s_vec[kHotWords];
+  __shared__ uint32_t s_host[kHotMax];
+  __shared__ uint32_t s_n;
+  const uint32_t tid = threadIdx.x;
+  const uint32_t tau_mask = (d.tau >= 32u) ? 0xFFFFFFFFu : ((1u << d.tau) - 1u);
+  const uint32_t wl = d.k_log2 - 5u;                               // log2 words of a vector
+  const uint32_t most = min(kHotMax, kHotWords >> wl);             // k <= 65,536: at least 2
+  const uint64_t head = (((uintptr_t)pairs & 15u) != 0u && n_pairs > 0) ? 1u : 0u;
+  const uint64_t body = (n_pairs - head) >> 1;                     // uint4 = 2 pairs
+  const uint4* p4 = reinterpret_cast<const uint4*>(pairs + 2 * head);
+  const uint64_t stride = (uint64_t)gridDim.x * kHotThreads;
+  uint64_t j = (uint64_t)blockIdx.x * kHotThreads + tid;
+  uint4 v = make_uint4(0u, 0u, 0u, 0u);
+  if (j < body) v = __ldcs(p4 + j);
+  for (uint32_t i = tid; i < kHotSlots; i += kHotThreads) s_tab[i] = make_uint2(kNoHost, 0u);
+  for (uint32_t i = tid; i < kHotWords; i += kHotThreads) s_vec[i] = 0u;
+  if (tid == 0) s_n = 0u;
+  __syncthreads();
+  auto slot_of = [](uint32_t hip) { return (hip * 0x9E3779B1u) >> 21; };   // kHotSlots = 2^11
+  auto sample = [&](uint32_t hip) {
+    if (hip == kNoHost) return;
+    uint2* s = &s_tab[slot_of(hip)];
+    const uint32_t was = atomicCAS(&s->x, kNoHost, hip);
+    if (was == kNoHost || was == hip) atomicAdd(&s->y, 1u);
+  };
+  if (j < body) {
+    sample(v.x);
+    sample(v.z);
+  }
+  __syncthreads();
+  for (uint32_t i = tid; i < kHotSlots; i += kHotThreads) {
+    uint32_t e = 0;
+    if (s_tab[i].y >= heavy) {
+      const uint32_t at = atomicAdd(&s_n, 1u);
+      if (at < most) {
+        s_host[at] = s_tab[i].x;
+        e = at + 1u;
+      }
+    }
+    s_tab[i].y = e;
+  }
+  __syncthreads();
+  auto pair = [&](uint32_t hip, uint32_t oip) {
+    const uint2 t = s_tab[slot_of(hip)];
+    if (t.x != hip || t.y == 0u) {
+      scan_pair<LR>(d, seav, ldca, hip, oip, tau_mask);
+      return;
+    }
+    const uint32_t h1 = mas(d.ha[0], d.hb[0], oip);
+    if ((h1 & tau_mask) == 0u) seav_update(d, seav, hip, h1);
+    const uint32_t h3 = mas(d.ha[1], d.hb[1], oip) >> (32u - d.k_log2);
+    atomicOr(&s_vec[((t.y - 1u) << wl) + (h3 >> 5)], 1u << (h3 & 31u));
+  };
+  while (j < body) {
+    const uint4 x = v;
+    j += stride;
+    if (j < body) v = __ldcs(p4 + j);
+    pair(x.x, x.y);
+    pair(x.z, x.w);
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    if (head) scan_pair<LR>(d, seav, ldca, pairs[0], pairs[1], tau_mask);
+    if ((n_pairs - head) & 1u) {
+      const uint64_t last = n_pairs - 1;
+      scan_pair<LR>(d, seav, ldca, pairs[2 * last], pairs[2 * last + 1], tau_mask);
+    }
+  }
+  __syncthreads();
+  const uint32_t held = min(s_n, most);
+  const uint32_t cshift = 32u - d.lc_log2;
+  for (uint32_t i = tid; i < held << wl; i += kHotThreads) {
+    const uint32_t bits = s_vec[i];
+    if (bits == 0u) continue;
+    const uint32_t hip = s_host[i >> wl], word = i & ((1u << wl) - 1u);
+#pragma unroll
+    for (int r = 0; r < LR; ++r) {
+      const uint32_t col = (uint32_t)((uint64_t)mas(d.ha[2 + r], d.hb[2 + r], hip) >> cshift);
+      atomicOr(ldca + ((((uint64_t)r << d.lc_log2 | col) << wl) | word), bits);
+    }
+  }
+}
+
 template <int LR>
 int grid_for() {
   int dev = 0, sms = 0, per_sm = 0;
@@ -205,20 +311,46 @@ int scan_grid(const DevParams& d) {
   }
 }
 
+namespace {
+
+// kHotPairs: at 2^18 pairs of mixed traffic (the heaviest host 1/8 of them)
+// k_scan takes 16.0 us and k_scan_hot 11.9, of uniform traffic 10.9 and 11.9;
+// at 2^17 11.9 both and 7.8 against 11.8.  At 2^20 64 against 26 us (mixed), 26
+// both (uniform).  Two blocks per SM: 3% faster than one from 2^20 on.
+template <int LR>
+void scan_launch(const DevParams& d, uint8_t* seav, uint32_t* ldca, const uint32_t* pairs, uint64_t n_pairs,
+                 int grid, cudaStream_t s) {
+  if (n_pairs < kHotPairs) {
+    k_scan<LR><<<grid, kScanThreads, 0, s>>>(d, seav, ldca, pairs, n_pairs);
+    return;
+  }
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const uint64_t need = (n_pairs / 2 + kHotThreads - 1) / kHotThreads;
+  const int blocks = need < (uint64_t)(2 * sms) ? (int)need : 2 * sms;
+  // a held host should have about 16 pairs in its block: heavy of the 2,048 sampled ones
+  const uint64_t per_block = n_pairs / (uint64_t)blocks;
+  const uint64_t heavy = 16u * 2048u / per_block;
+  k_scan_hot<LR><<<blocks, kHotThreads, 0, s>>>(d, seav, ldca, pairs, n_pairs, (uint32_t)(heavy < 4 ? 4 : heavy));
+}
+
+}  // namespace
+
 cudaError_t launch_scan(const DevParams& d, uint8_t* seav, uint32_t* ldca,
                         const uint32_t* pairs, uint64_t n_pairs, int grid, cudaStream_t s) {
   if (n_pairs == 0) return cudaSuccess;
   const uint64_t need = (n_pairs / 2 + kScanThreads - 1) / kScanThreads;
   if ((uint64_t)grid > need) grid = (int)(need > 0 ? need : 1);
   switch (d.lr) {
-    case 1: k_scan<1><<<grid, kScanThreads, 0, s>>>(d, seav, ldca, pairs, n_pairs); break;
-    case 2: k_scan<2><<<grid, kScanThreads, 0, s>>>(d, seav, ldca, pairs, n_pairs); break;
-    case 3: k_scan<3><<<grid, kScanThreads, 0, s>>>(d, seav, ldca, pairs, n_pairs); break;
-    case 4: k_scan<4><<<grid, kScanThreads, 0, s>>>(d, seav, ldca, pairs, n_pairs); break;
-    case 5: k_scan<5><<<grid, kScanThreads, 0, s>>>(d, seav, ldca, pairs, n_pairs); break;
-    case 6: k_scan<6><<<grid, kScanThreads, 0, s>>>(d, seav, ldca, pairs, n_pairs); break;
-    case 7: k_scan<7><<<grid, kScanThreads, 0, s>>>(d, seav, ldca, pairs, n_pairs); break;
-    default: k_scan<8><<<grid, kScanThreads, 0, s>>>(d, seav, ldca, pairs, n_pairs); break;
+    case 1: scan_launch<1>(d, seav, ldca, pairs, n_pairs, grid, s); break;
+    case 2: scan_launch<2>(d, seav, ldca, pairs, n_pairs, grid, s); break;
+    case 3: scan_launch<3>(d, seav, ldca, pairs, n_pairs, grid, s); break;
+    case 4: scan_launch<4>(d, seav, ldca, pairs, n_pairs, grid, s); break;
+    case 5: scan_launch<5>(d, seav, ldca, pairs, n_pairs, grid, s); break;
+    case 6: scan_launch<6>(d, seav, ldca, pairs, n_pairs, grid, s); break;
+    case 7: scan_launch<7>(d, seav, ldca, pairs, n_pairs, grid, s); break;
+    default: scan_launch<8>(d, seav, ldca, pairs, n_pairs, grid, s); break;
   }
   return cudaGetLastError();
 }
