@@ -25,9 +25,9 @@
 //   sp_candidate records with est taken from a table of -k ln(z0 / k).  Up to
 //   2,048 keys one block sorts them in shared memory (bitonic).  Above that,
 //   the cooperative grid sorts runs of 2,048 keys in shared memory, one block
-//   per run, then merges groups of 16 runs per round between grid-wide
+//   per run, then merges groups of up to 8 runs per round between grid-wide
 //   barriers: each key's place in the merged run is its index in its own run
-//   plus the number of keys of the other 15 runs below it (binary searches
+//   plus the number of keys of the group's other runs below it (binary searches
 //   side by side).  The rounds alternate between the key buffer and the record
 //   buffer (which holds at least as many bytes); the last one reads the key
 //   buffer and writes the records.
@@ -398,7 +398,7 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
 // ---- sort + emit ----------------------------------------------------------
 constexpr int kSortThreads = 1024;
 constexpr uint32_t kRun = 2048;           // keys one block sorts in shared memory (16 KiB, two per thread)
-constexpr int kWays = 16;                 // runs merged per round
+constexpr int kWays = 8;                  // runs merged per round, at most
 
 __device__ __forceinline__ void emit_record(uint64_t key, const double* est_table, sp_candidate* out) {
   sp_candidate c;
@@ -434,33 +434,53 @@ __device__ void smem_bitonic(uint64_t* a, uint32_t m) {
   __syncthreads();
 }
 
-// Place of a key within its group of kWays runs of w keys (a power of two;
-// group = [base, end) of src, only its last run may be shorter): its index in
-// its own run plus the keys of every other run below it.  The searches of the
-// runs advance together, so a step costs one memory round trip for all.
+// Place of a key within its group of WAYS runs of w keys (a power of two;
+// group = [base, end) of src, only its last run may be shorter): the keys of
+// every run below it (its index, in its own).  The searches of the
+// runs advance together, so a step costs one memory round trip for all; ips are
+// unique, so a step compares the keys' upper words.
+template <int WAYS>
 __device__ __forceinline__ uint32_t merged_place(const uint64_t* src, uint32_t base, uint32_t end, uint32_t w,
-                                                 uint32_t i, uint64_t key) {
-  const uint32_t own = (i - base) / w;
-  uint32_t pos[kWays];
+                                                 uint64_t key) {
+  const uint32_t ip = (uint32_t)(key >> 32);
+  const uint32_t* ips = reinterpret_cast<const uint32_t*>(src) + 1;       // ips[2 g] = ip of key g
+  uint32_t pos[WAYS];
 #pragma unroll
-  for (int q = 0; q < kWays; ++q) pos[q] = 0;
+  for (int q = 0; q < WAYS; ++q) pos[q] = 0;
   // after steps w, w / 2, ..., 1: pos[q] = keys of run q below key
   for (uint32_t step = w; step > 0; step >>= 1) {
 #pragma unroll
-    for (int q = 0; q < kWays; ++q) {
+    for (int q = 0; q < WAYS; ++q) {
       const uint32_t at = pos[q] + step;                           // 1-based rank tried
       const uint64_t g = (uint64_t)base + (uint64_t)q * w + at - 1;
-      if (at <= w && g < end && (uint32_t)q != own && src[g] < key) pos[q] = at;
+      if (at <= w && g < end && ips[2 * g] < ip) pos[q] = at;
     }
   }
-  uint32_t place = i - own * w;                                    // base + index in the own run
+  uint32_t place = base;                                           // the own run counts the key's index in it
 #pragma unroll
-  for (int q = 0; q < kWays; ++q) place += pos[q];
+  for (int q = 0; q < WAYS; ++q) place += pos[q];
   return place;
 }
 
+// one merge round: groups of WAYS runs of w keys, to dst or (out != null) to the records
+template <int WAYS>
+__device__ __forceinline__ void merge_round(const uint64_t* src, uint64_t* dst, sp_candidate* out,
+                                            const double* est_table, uint64_t n, uint64_t w) {
+  const uint64_t group = w * WAYS;
+  for (uint64_t i = (uint64_t)blockIdx.x * kSortThreads + threadIdx.x; i < n; i += (uint64_t)gridDim.x * kSortThreads) {
+    const uint64_t base = i / group * group;
+    const uint64_t end = base + group < n ? base + group : n;
+    const uint64_t key = src[i];
+    const uint32_t place = merged_place<WAYS>(src, (uint32_t)base, (uint32_t)end, (uint32_t)w, key);
+    if (out) emit_record(key, est_table, out + place);
+    else dst[place] = key;
+  }
+}
+
 // Bounds: latency.  Up to kRun keys: 66 stages in one block (4.4 us at ~500
-// keys).  Above: one run per block, then ceil(log16(runs)) merge rounds.
+// keys).  Above: one run per block, then ceil(log8(runs)) merge rounds; 8 ways
+// because a key's searches are then bound by their round trips, not by their
+// instructions (a detect with 150,000 results: 234 us with 16 ways, 195 with 8).
 __global__ void __launch_bounds__(kSortThreads)
 k_sort_emit(uint64_t* keys, uint32_t cap, const DetectStatus* status, const double* est_table,
             sp_candidate* out) {
@@ -496,20 +516,13 @@ k_sort_emit(uint64_t* keys, uint32_t cap, const DetectStatus* status, const doub
     __syncthreads();
   }
   // 2. merge rounds; the last one reads the key buffer and writes the records
-  const uint64_t gtid = (uint64_t)blockIdx.x * kSortThreads + tid;
-  const uint64_t gsize = (uint64_t)gridDim.x * kSortThreads;
   for (uint64_t w = kRun; w < n; w *= kWays) {
     grid.sync();
-    const uint64_t group = w * kWays;
-    const bool last = group >= n;
-    for (uint64_t i = gtid; i < n; i += gsize) {
-      const uint64_t base = i / group * group;
-      const uint64_t end = base + group < n ? base + group : n;
-      const uint64_t key = src[i];
-      const uint32_t place = merged_place(src, (uint32_t)base, (uint32_t)end, (uint32_t)w, (uint32_t)i, key);
-      if (last) emit_record(key, est_table, out + place);
-      else dst[place] = key;
-    }
+    const uint64_t left = (n + w - 1) / w;                         // runs
+    sp_candidate* to = left <= kWays ? out : nullptr;
+    if (left <= 2) merge_round<2>(src, dst, to, est_table, n, w);
+    else if (left <= 4) merge_round<4>(src, dst, to, est_table, n, w);
+    else merge_round<kWays>(src, dst, to, est_table, n, w);
     uint64_t* t = src;
     src = dst;
     dst = t;
