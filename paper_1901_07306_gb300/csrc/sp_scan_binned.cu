@@ -387,17 +387,21 @@ __device__ __forceinline__ uint4 load_hips(const uint32_t* p) {
 // a plane, each holding LR / SPLIT of its LDCA rows in shared memory and
 // reading the whole hip list: wide planes (LC = 2^18: 128 KiB for four rows)
 // would otherwise leave one block per SM.
-// Groups of 8 lanes walk the plane's lists on their own, 32 hips a step, one
-// 16-byte load per lane, issued a step ahead, so that short lists -- a launch
-// of 5 M pairs leaves 32 hips in each -- cost one load's latency for the whole
-// plane and not one count and one load per list and warp; the lists' counts
-// are in shared memory before the walk starts.  A group takes whole lists:
-// sharing one among 2 or 4 groups balances the warps better and measured 3%
-// slower (more ragged ends), two loads per lane and step the same.
+// Groups of 8 lanes walk the plane's lists on their own (list c, c + NG, ...),
+// 2 x 32 hips a step, two 16-byte loads per lane, issued a step ahead and the
+// first step before the plane is zeroed: short lists -- a launch of 5 M pairs
+// leaves 32 hips in each, one of 2^24 108 -- are bound by the loads' latency.
+// The lists' counts are in shared memory before the walk starts.  A group takes
+// whole lists: sharing one among 2 or 4 groups balances the warps better and
+// measured 3% slower (more ragged ends).  Two loads a step at three blocks per
+// SM (40 registers): 16 routers x 2^24 pairs scan in 2.33 ms against 2.49 with
+// one load, and 2^26 pairs in 333 against 336 us; at four blocks (32
+// registers, spills) 2.33 ms and 344 us.
 // Lists are filled up to whole 8-hip chunks (k_bin), so a lane's 4 hips are
 // all there or none is.
+constexpr int kQuads = 2;
 template <int LR, int THREADS, int LCL, int SPLIT>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, 1536 / THREADS)
 k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restrict__ counts,
         uint32_t G, uint32_t cap, const uint32_t* planes, const __grid_constant__ CUtensorMap map, uint32_t box,
         bool accumulate) {
@@ -410,6 +414,20 @@ k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restr
   const uint32_t chunks = ((((uint32_t)LRP << lc_log2) >> 5) + 7u) / 8u;  // 8-word chunks of the block's rows
   uint32_t* s_count = s_plane + chunks * 8u;                       // [G]
   const uint32_t tid = threadIdx.x, lane = tid & 31u;
+  const uint32_t first = 4u * (lane & 7u);                          // this lane's hips of a step
+  uint32_t c = tid >> 3, at = first;
+  counts += (uint64_t)b * G;
+  uint32_t n = c < G ? counts[c] : 0u;
+  const uint32_t* list = lists + ((uint64_t)b * G + c) * cap;
+  struct Step { uint4 h[kQuads]; uint32_t have; };                 // have: valid 16-byte loads
+  auto load = [&](Step& s) {
+    s.have = at < n ? min((n - at + 31u) / 32u, (uint32_t)kQuads) : 0u;
+#pragma unroll
+    for (int u = 0; u < kQuads; ++u)
+      if ((uint32_t)u < s.have) s.h[u] = load_hips<SPLIT>(list + at + 32 * u);
+  };
+  Step s0, s1;
+  load(s0);
   // LH_i(hip) = h >> cshift (5 <= lc_log2 <= 20): LDC h >> cshift of row i is
   // bit (h >> cshift) mod 32 of plane word (i << (lc_log2 - 5)) + (h >> (cshift + 5))
   const uint32_t cshift = 32u - lc_log2;
@@ -429,7 +447,7 @@ k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restr
     a_hi[r] = (uint32_t)(d.ha[2 + row0 + r] >> 32);
     bw[r] = d.hb[2 + row0 + r];
   }
-  for (uint32_t c = tid; c < G; c += THREADS) s_count[c] = counts[(uint64_t)b * G + c];
+  for (uint32_t i = tid; i < G; i += THREADS) s_count[i] = counts[i];
   for (uint32_t u = tid; u < chunks * 2u; u += THREADS)             // 16-byte units, consecutive lanes
     *reinterpret_cast<uint4*>(s_plane + u * 4u) =
         accumulate ? *reinterpret_cast<const uint4*>(src + (u >> 1) * chunk_stride + (u & 1u) * 4u)
@@ -450,35 +468,29 @@ k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restr
       }
     }
   };
-  const uint32_t first = 4u * (lane & 7u);                          // this lane's hips of a step: first .. first + 3
-  uint32_t c = tid >> 3, at = first;
-  uint32_t n = c < G ? s_count[c] : 0u;
-  const uint32_t* list = lists + ((uint64_t)b * G + c) * cap;
-  uint4 cur = make_uint4(0u, 0u, 0u, 0u);
-  bool have = at < n;
-  if (have) cur = load_hips<SPLIT>(list + at);
-  bool live = c < G;
-  while (__any_sync(kFull, live)) {
-    at += 32u;
+  // loads the next step, then sets the bits of the current one; false when no
+  // group of the warp has a list left
+  auto turn = [&](Step& cur, Step& next) {
+    if (!__any_sync(kFull, c < G)) return false;
+    at += 32u * kQuads;
     if (at - first >= n) {                                          // the group's next list
       c += NG;
       at = first;
       n = c < G ? s_count[c] : 0u;
       list += (uint64_t)NG * cap;
     }
-    live = c < G;
-    const bool more = at < n;
-    uint4 next = cur;
-    if (more) next = load_hips<SPLIT>(list + at);
-    if (have) {
-      set_bits(cur.x);
-      set_bits(cur.y);
-      set_bits(cur.z);
-      set_bits(cur.w);
-    }
-    cur = next;
-    have = more;
-  }
+    load(next);
+#pragma unroll
+    for (int u = 0; u < kQuads; ++u)
+      if ((uint32_t)u < cur.have) {
+        set_bits(cur.h[u].x);
+        set_bits(cur.h[u].y);
+        set_bits(cur.h[u].z);
+        set_bits(cur.h[u].w);
+      }
+    return true;
+  };
+  while (turn(s0, s1) && turn(s1, s0)) {}
   // the plane's chunks go out by TMA, `box` chunks a copy: 1,024 sectors 32 KiB
   // apart (profile D), which as 32-byte stores took one wavefront of the
   // load-store pipe each, the pipe that bounds the kernel
