@@ -12,8 +12,9 @@
 //           stages each hip in a shared-memory row of its bin b; a row's whole
 //           8-hip chunks go to the block's private list for that bin with one
 //           32-byte store each (no global atomics; lists[b][block][0 .. cap)).
-//           A row or a list that is full sends its hips to L2 REDs instead
-//           (any input is correct; only a skewed one is slower).
+//           Hips that find their row full wait for the end of the round; only
+//           skewed inputs (a full list, a row that stays full) send hips to L2
+//           REDs instead (any input is correct).
 //  k_apply  (one block per plane) starts the plane in shared memory from
 //           zero (or from the router's pending plane when earlier updates of
 //           the window have not been folded yet), sets bit (i, LH_i(hip)) for
@@ -48,6 +49,7 @@ namespace {
 constexpr int kVec = 4;                            // 16-byte loads (2 pairs) per thread and tile
 constexpr int kGroup = 4;                          // pairs hashed and staged together
 constexpr int kChunk = 8;                          // hips per list store (32 bytes)
+constexpr int kOver = 128;                         // pairs per round that found their row full
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 
 __device__ __forceinline__ void seav_set(const DevParams& d, uint8_t* seav, uint32_t hip, uint32_t h1) {
@@ -91,8 +93,10 @@ __device__ __forceinline__ void st_chunk(uint32_t* dst, uint4 a, uint4 b) {
 // write-combining buffer for the bin's list).  Per tile:
 //   1. every thread hashes its pairs, queues the sampled pairs (Sec. 3.1) for
 //      a converged SEAV pass, takes a place in its pair's bin row with one
-//      shared atomic and stores the hip there (a row that is full sends the
-//      pair to L2 REDs instead);
+//      shared atomic and stores the hip there (of a row that is full, which 2 in
+//      a million are by chance, the pair waits for the end of the round: a
+//      single LDCA bit set past the lists would make the fold read 32 MiB of
+//      LDCA, the merge 128 MiB per router of profile D3 and the reset zero them);
 //   2. (after every TPR tiles) each thread takes bins tid, tid + THREADS, ...:
 //      it moves the row's whole 8-hip chunks to the bin's list with 32-byte
 //      stores and keeps the remainder (< 8 hips) at the front of the row; the
@@ -113,9 +117,10 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
   uint32_t* stage = reinterpret_cast<uint32_t*>(smem_raw);             // [bins][STAGE], then a 32-word sink
   uint32_t* sink = stage + bins * STAGE;                                // stores of pairs a full row refused
   uint2* s_queue = reinterpret_cast<uint2*>(sink + 32);               // [QUEUE] sampled (hip, h1)
-  uint32_t* s_fill = reinterpret_cast<uint32_t*>(s_queue + QUEUE);     // [bins] hips in the row
+  uint2* s_over = s_queue + QUEUE;                                      // [2][kOver] (hip, bin) of full rows, by round parity
+  uint32_t* s_fill = reinterpret_cast<uint32_t*>(s_over + 2 * kOver);  // [bins] hips in the row
   uint32_t* s_cursor = s_fill + bins;                                   // [bins] list fill (whole chunks)
-  __shared__ uint32_t s_qn[2];                                          // queue fill, by tile parity
+  __shared__ uint32_t s_qn[2], s_on[2];                                 // queue and s_over fill, by round parity
   __shared__ uint32_t s_full[kBinMaxSrc + 1], s_small[kBinMaxSrc + 1];   // tiles before stream b (fewer than 2^32 a round)
   const uint32_t tid = threadIdx.x;
   const uint32_t G = gridDim.x, cta = blockIdx.x;
@@ -161,7 +166,7 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
 #pragma unroll
     for (int e = 0; e < kBinMaxSrc / 32; ++e) pref[lane * (kBinMaxSrc / 32) + (uint32_t)e + 1] = incl - acc + sum[e];
     if (lane == 0) pref[0] = 0;
-    if (tid == 0) s_qn[0] = s_qn[1] = 0;
+    if (tid == 0) s_qn[0] = s_qn[1] = s_on[0] = s_on[1] = 0;
   }
   auto list_of = [&](uint32_t b) { return lists + ((uint64_t)b * G + cta) * cap; };
   for (uint32_t b = tid; b < bins; b += THREADS) {
@@ -221,14 +226,19 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
     }
     return over;
   };
-  // the rare leftovers of a group: pairs whose row was full (LDCA bits with
-  // L2 REDs) and sampled pairs the full queue did not take (SEAV bits)
+  // the rare leftovers of a group: pairs whose row was full wait in s_over for
+  // the end of the round (LDCA bits with L2 REDs only when that is full too),
+  // sampled pairs the full queue did not take set their SEAV bits
   auto group_leftovers = [&](const uint32_t (&hip)[kGroup], const uint32_t (&oip)[kGroup],
-                             const uint32_t (&bin)[kGroup], uint32_t over) {
+                             const uint32_t (&bin)[kGroup], uint32_t over, uint32_t par) {
     if (__any_sync(kFull, over != 0u)) {
 #pragma unroll
       for (int q = 0; q < kGroup; ++q) {
-        if ((over >> q) & 1u) spill(hip[q], bin[q]);
+        if ((over >> q) & 1u) {
+          const uint32_t at = atomicAdd(&s_on[par], 1u);
+          if (at < (uint32_t)kOver) s_over[par * kOver + at] = make_uint2(hip[q], bin[q]);
+          else spill(hip[q], bin[q]);
+        }
         if ((over >> (kGroup + q)) & 1u) seav_set(d, seav, hip[q], mas(d.ha[0], d.hb[0], oip[q]));
       }
     }
@@ -268,7 +278,7 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
         hip[2 * u + 1] = v.z; oip[2 * u + 1] = v.w;
       }
       const uint32_t over = stage_group(hip, oip, (1u << kGroup) - 1u, par, bin);
-      group_leftovers(hip, oip, bin, over);
+      group_leftovers(hip, oip, bin, over, par);
     }
   };
   // the flush round: whole chunks to the lists; the queued SEAV updates,
@@ -276,7 +286,8 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
   auto flush_round = [&](uint32_t par) {
     __syncthreads();
     const uint32_t qn = s_qn[par] < (uint32_t)QUEUE ? s_qn[par] : (uint32_t)QUEUE;
-    if (tid == 0) s_qn[par ^ 1u] = 0;            // read by every thread before the last barrier
+    const uint32_t on = s_on[par] < (uint32_t)kOver ? s_on[par] : (uint32_t)kOver;
+    if (tid == 0) s_qn[par ^ 1u] = s_on[par ^ 1u] = 0;   // read by every thread before the last barrier
     for (uint32_t b = tid; b < bins; b += THREADS) {
       const uint32_t f = s_fill[b];
       if (f >= (uint32_t)kChunk) flush_row(b, f < (uint32_t)STAGE ? f : (uint32_t)STAGE);
@@ -286,6 +297,13 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
       seav_set(d, seav, x.x, x.y);
     }
     __syncthreads();
+    // the round's leftovers take places in the rows, which have room again
+    if (tid < on) {
+      const uint2 x = s_over[par * kOver + tid];
+      const uint32_t at = atomicAdd(&s_fill[x.y], 1u);
+      if (at < (uint32_t)STAGE) stage[x.y * STAGE + at] = x.x;
+      else spill(x.x, x.y);
+    }
   };
   // Tiles in pairs (i, i + 1) in the two register buffers.  A buffer's loads
   // for tile t + 2 go out as soon as tile t is staged, so the flush round
@@ -348,11 +366,17 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
       }
       if (__any_sync(kFull, valid != 0u)) {
         const uint32_t over = stage_group(hip, oip, valid, par, bin);
-        group_leftovers(hip, oip, bin, over);
+        group_leftovers(hip, oip, bin, over, par);
       }
     }
     flush_round(par);
     par ^= 1u;
+  }
+  // the last round's leftovers are in the rows: whole chunks once more
+  __syncthreads();
+  for (uint32_t b = tid; b < bins; b += THREADS) {
+    const uint32_t f = s_fill[b];
+    if (f >= (uint32_t)kChunk) flush_row(b, f < (uint32_t)STAGE ? f : (uint32_t)STAGE);
   }
   // remainders (< 8 hips per row): one more chunk, filled up with copies of a
   // hip of its own, so that k_apply reads whole 16-byte quads of a list (a bit
@@ -726,8 +750,8 @@ template <int THREADS, int STAGE, int TPR, int PER_SM>
 cudaError_t bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, const BinSrc& src,
                       const BinnedScratch& s, uint32_t cap, bool append, uint32_t rot, cudaStream_t st) {
   const uint32_t bins = 1u << d.k_log2;
-  // the bins' staging rows, the sampled-pair queue, 2 counters per bin
-  const size_t bin_smem = (size_t)bins * STAGE * 4 + 32 * 4 + (size_t)(TPR * THREADS * kVec * 2 / 32) * 8 +
+  // the bins' staging rows, the sampled-pair queue, the full rows' pairs, 2 counters per bin
+  const size_t bin_smem = (size_t)bins * STAGE * 4 + 32 * 4 + (size_t)(TPR * THREADS * kVec * 2 / 32 + 2 * kOver) * 8 +
                           (size_t)bins * 8;
   auto kern = k_bin<THREADS, STAGE, TPR, PER_SM>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bin_smem);

@@ -56,3 +56,25 @@ def test_many_odd_streams_in_a_launch(sp, torch):  # noqa: F811
     with sp.SuperPoint(**kw) as ctx:
         sp.sp_update_batched(ctx.ctx, [0] * len(parts), [dev(torch, p, i & 1) for i, p in enumerate(parts)])
         assert_same_sketch(ctx, O.Sketch(oracle_params(kw)).update(np.concatenate(parts)))
+
+
+@pytest.mark.parametrize("shape", [0, 2])
+@pytest.mark.parametrize("peers", [2, 300, 500, 700])
+def test_rows_that_overflow(sp, torch, peers, shape):  # noqa: F811
+    """Few distinct peers crowd few bins: rows overflow now and then (the pairs
+    wait for the end of the round) or all the time (L2 REDs)."""
+    kw = dict(KW, k_log2=10, lr=4, lc_log2=12, theta=8, n_routers=2)
+    rng = np.random.default_rng(peers)
+    n = 2 * ROUND + 12345
+    oips = rng.integers(0, 2**32, peers, dtype=np.uint32)
+    x = np.stack([rng.integers(0, 2**32, n, dtype=np.uint32), oips[rng.integers(0, peers, n)]], 1)
+    with sp.SuperPoint(**kw) as ctx:
+        sp.sp_set_binned_shape(ctx.ctx, shape)
+        ctx.update(dev(torch, x))
+        osk = O.Sketch(oracle_params(kw)).update(x)
+        ctx.merge([0], 1)
+        assert_same_sketch(ctx, osk, 1)
+        assert_same_sketch(ctx, osk, 0)
+        ctx.reset(0)
+        seav, ldca = ctx.sketch_image(0)
+        assert not seav.any() and not ldca.any()
