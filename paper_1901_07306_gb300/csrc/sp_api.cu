@@ -28,7 +28,8 @@ constexpr uint64_t kBinnedRoundPairs = 1ull << 26;  // pairs per binning round
 // Host-path binning rounds: each round's plane pass overlaps the next round's
 // copies, so after the last copy only one round of 2^24 pairs is left to apply.
 constexpr uint64_t kHostRoundPairs = 1ull << 24;
-constexpr uint32_t kResultPrefix = 4096;            // records fetched with the status
+constexpr uint32_t kResultPrefix = 2048;            // records fetched with the status (48 KiB)
+constexpr size_t kKerrAt = 64, kRecordsAt = 128;    // result block: status, error word, records
 constexpr uint32_t kDefaultTimeoutMs = 60000;       // bound of every wait on the stream
 constexpr uint64_t kAlign = 256;
 
@@ -90,9 +91,15 @@ struct sp_ctx {
   uint64_t seav_bytes = 0, ldca_bytes = 0, seav_pad = 0, stride = 0;
   uint8_t* sketches = nullptr;              // n_routers * stride bytes
   uint64_t* keys = nullptr;                 // detect scratch: next_pow2(cap) keys
-  sp_candidate* records = nullptr;          // sorted results, cap records
-  DetectStatus* status = nullptr;
-  uint32_t* kerr = nullptr;                 // kernel error word (bad device batch table entries)
+  // the result block: the last detect's status, the kernel error word (bad
+  // device batch table entries) and the sorted records, one behind the other
+  // so that one copy fetches what a small result needs
+  uint8_t* results = nullptr;
+  DetectStatus* published() const { return reinterpret_cast<DetectStatus*>(results); }
+  uint32_t* kerr() const { return reinterpret_cast<uint32_t*>(results + kKerrAt); }
+  sp_candidate* records() const { return reinterpret_cast<sp_candidate*>(results + kRecordsAt); }
+  DetectStatus* status = nullptr;           // the running detect's; zero between detects
+  bool status_clean = true;                 // false: a detect's second launch failed
   double* est_table = nullptr;              // -k ln(z / k), z = 0 .. k
   uint32_t cap = 0;
   uint32_t timeout_ms = kDefaultTimeoutMs;  // 0: waits are unbounded
@@ -359,9 +366,8 @@ void sp_destroy(sp_ctx* ctx) {
   free(ctx->ldca_zero);
   cudaFree(ctx->sketches);
   cudaFree(ctx->keys);
-  cudaFree(ctx->records);
+  cudaFree(ctx->results);
   cudaFree(ctx->status);
-  cudaFree(ctx->kerr);
   cudaFree(ctx->est_table);
   if (ctx->ev_wait) cudaEventDestroy(ctx->ev_wait);
   if (ctx->ev_arena) cudaEventDestroy(ctx->ev_arena);
@@ -414,9 +420,8 @@ int sp_create(const sp_params* p, void* cuda_stream, sp_ctx** out) {
   int rc = SP_OK;
   if (cudaMalloc(&c->sketches, c->stride * p->n_routers) != cudaSuccess ||
       cudaMalloc(&c->keys, key_slots * sizeof(uint64_t)) != cudaSuccess ||
-      cudaMalloc(&c->records, (uint64_t)c->cap * sizeof(sp_candidate)) != cudaSuccess ||
+      cudaMalloc(&c->results, kRecordsAt + (uint64_t)c->cap * sizeof(sp_candidate)) != cudaSuccess ||
       cudaMalloc(&c->status, sizeof(DetectStatus)) != cudaSuccess ||
-      cudaMalloc(&c->kerr, sizeof(uint32_t)) != cudaSuccess ||
       cudaMalloc(&c->ovf, sizeof(uint32_t) * p->n_routers) != cudaSuccess ||
       cudaMalloc(&c->est_table, ((1ull << p->k_log2) + 1) * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
@@ -439,7 +444,7 @@ int sp_create(const sp_params* p, void* cuda_stream, sp_ctx** out) {
                          cudaSuccess)
     rc = SP_ERR_CUDA;
   if (rc == SP_OK && cudaMemsetAsync(c->status, 0, sizeof(DetectStatus), c->stream) != cudaSuccess) rc = SP_ERR_CUDA;
-  if (rc == SP_OK && cudaMemsetAsync(c->kerr, 0, sizeof(uint32_t), c->stream) != cudaSuccess) rc = SP_ERR_CUDA;
+  if (rc == SP_OK && cudaMemsetAsync(c->results, 0, kRecordsAt, c->stream) != cudaSuccess) rc = SP_ERR_CUDA;
   if (rc == SP_OK) {
     c->scan_grid = sp::scan_grid(d);
     c->multi_grid = sp::multi_max_grid(c->multi_threads);
@@ -824,7 +829,7 @@ static int launch_table(sp_ctx* ctx, const sp_batch* dev_tab, uint32_t n) {
   for (uint32_t i = 0; i < n; i += kMaxTable) {
     const uint32_t m = (n - i) < kMaxTable ? (n - i) : kMaxTable;
     if (sp::launch_scan_multi(ctx->d, ctx->sketches, ctx->stride, ctx->seav_pad, ctx->p.n_routers, dev_tab + i, m,
-                              ctx->kerr, ctx->multi_threads, ctx->multi_grid, ctx->stream) != cudaSuccess)
+                              ctx->kerr(), ctx->multi_threads, ctx->multi_grid, ctx->stream) != cudaSuccess)
       return SP_ERR_CUDA;
   }
   return SP_OK;
@@ -1179,7 +1184,10 @@ int sp_detect_async(sp_ctx* ctx, uint32_t router, uint32_t threshold) {
   const uint32_t zt = sp_z_theta(ctx->p.k_log2, threshold);
   int frc = ctx->sliding ? commit_seav_window(ctx, router) : fold_router(ctx, router);
   if (frc != SP_OK) return frc;
-  if (cudaMemsetAsync(ctx->status, 0, sizeof(DetectStatus), ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
+  // the status is zero here: each detect's last kernel leaves it so
+  if (!ctx->status_clean && cudaMemsetAsync(ctx->status, 0, sizeof(DetectStatus), ctx->stream) != cudaSuccess)
+    return SP_ERR_CUDA;
+  ctx->status_clean = false;
   // a sliding router is detected on its window SEAV and, for the LDCA test of
   // each tested host, the active stamps and pending slice bits of its lines
   const cudaError_t de =
@@ -1191,7 +1199,8 @@ int sp_detect_async(sp_ctx* ctx, uint32_t router, uint32_t threshold) {
                               ctx->p.max_join, ctx->status, ctx->stream);
   if (de != cudaSuccess) return SP_ERR_CUDA;
   if (sp::launch_sort_emit(ctx->keys, ctx->cap, ctx->status, ctx->est_table, ctx->p.k_log2,
-                           ctx->records, ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
+                           ctx->records(), ctx->published(), ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
+  ctx->status_clean = true;
   ctx->detect_issued = true;
   ctx->last_threshold = threshold;
   return threshold < ctx->p.theta ? SP_WARN_THETA_BELOW_INIT : SP_OK;
@@ -1200,22 +1209,18 @@ int sp_detect_async(sp_ctx* ctx, uint32_t router, uint32_t threshold) {
 int sp_results(sp_ctx* ctx, sp_candidate* host_out, uint64_t cap, uint64_t* n_total) {
   if (!ctx || !n_total || (cap && !host_out)) return SP_ERR_PARAM;
   if (!ctx->detect_issued) return SP_ERR_STATE;
-  // status, error word and a prefix of the records come back with one wait
-  constexpr size_t kKerrAt = 64, kRecordsAt = 128;
-  static_assert(sizeof(DetectStatus) <= kKerrAt, "status slot");
+  // status, error word and a prefix of the records come back with one copy and one wait
+  static_assert(sizeof(DetectStatus) <= kKerrAt && sizeof(uint32_t) <= kRecordsAt - kKerrAt, "result block");
   if (!ctx->result_host &&
       cudaMallocHost(&ctx->result_host, kRecordsAt + (size_t)kResultPrefix * sizeof(sp_candidate)) != cudaSuccess) {
     cudaGetLastError();
     ctx->result_host = nullptr;
     return SP_ERR_NOMEM;
   }
-  const uint64_t pre = ctx->cap < kResultPrefix ? ctx->cap : kResultPrefix;
-  if (cudaMemcpyAsync(ctx->result_host, ctx->status, sizeof(DetectStatus), cudaMemcpyDeviceToHost,
-                      ctx->stream) != cudaSuccess ||
-      cudaMemcpyAsync(ctx->result_host + kKerrAt, ctx->kerr, sizeof(uint32_t), cudaMemcpyDeviceToHost,
-                      ctx->stream) != cudaSuccess ||
-      (pre && cudaMemcpyAsync(ctx->result_host + kRecordsAt, ctx->records, pre * sizeof(sp_candidate),
-                              cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess)) return SP_ERR_CUDA;
+  uint64_t pre = ctx->cap < kResultPrefix ? ctx->cap : kResultPrefix;
+  if (cap < pre) pre = cap;
+  if (cudaMemcpyAsync(ctx->result_host, ctx->results, kRecordsAt + pre * sizeof(sp_candidate), cudaMemcpyDeviceToHost,
+                      ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
   int wrc = wait_stream(ctx);
   if (wrc != SP_OK) return wrc;
   DetectStatus st;
@@ -1224,7 +1229,7 @@ int sp_results(sp_ctx* ctx, sp_candidate* host_out, uint64_t cap, uint64_t* n_to
   memcpy(&kerr, ctx->result_host + kKerrAt, sizeof(kerr));
   if (kerr) {
     // a device batch table named a bad router or stream (the batch was skipped)
-    cudaMemsetAsync(ctx->kerr, 0, sizeof(uint32_t), ctx->stream);
+    cudaMemsetAsync(ctx->kerr(), 0, sizeof(uint32_t), ctx->stream);
     *n_total = st.count;
     return SP_ERR_ROUTER;
   }
@@ -1234,7 +1239,7 @@ int sp_results(sp_ctx* ctx, sp_candidate* host_out, uint64_t cap, uint64_t* n_to
   const uint64_t staged = m < pre ? m : pre;
   if (staged) memcpy(host_out, ctx->result_host + kRecordsAt, staged * sizeof(sp_candidate));
   if (m > staged) {
-    if (cudaMemcpyAsync(host_out + staged, ctx->records + staged, (m - staged) * sizeof(sp_candidate),
+    if (cudaMemcpyAsync(host_out + staged, ctx->records() + staged, (m - staged) * sizeof(sp_candidate),
                         cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
     if ((wrc = wait_stream(ctx)) != SP_OK) return wrc;
   }
@@ -1247,9 +1252,9 @@ int sp_results_async(sp_ctx* ctx, sp_candidate* host_out, uint64_t cap, uint32_t
   if (!ctx || !host_status || (cap && !host_out)) return SP_ERR_PARAM;
   if (!ctx->detect_issued) return SP_ERR_STATE;
   const uint64_t m = cap < ctx->cap ? cap : ctx->cap;
-  if (cudaMemcpyAsync(host_status, ctx->status, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess)
+  if (cudaMemcpyAsync(host_status, ctx->published(), 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess)
     return SP_ERR_CUDA;
-  if (m && cudaMemcpyAsync(host_out, ctx->records, m * sizeof(sp_candidate), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess)
+  if (m && cudaMemcpyAsync(host_out, ctx->records(), m * sizeof(sp_candidate), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess)
     return SP_ERR_CUDA;
   return SP_OK;
 }
@@ -1264,8 +1269,8 @@ int sp_detect(sp_ctx* ctx, uint32_t router, uint32_t threshold,
 
 int sp_results_device(sp_ctx* ctx, const sp_candidate** dev_records, const uint32_t** dev_count) {
   if (!ctx || !dev_records || !dev_count) return SP_ERR_PARAM;
-  *dev_records = ctx->records;
-  *dev_count = &ctx->status->count;
+  *dev_records = ctx->records();
+  *dev_count = &ctx->published()->count;
   return SP_OK;
 }
 

@@ -33,6 +33,8 @@
 //   buffer and writes the records.
 #include <cooperative_groups.h>
 
+#include <atomic>
+
 #include "sp_internal.h"
 
 namespace cg = cooperative_groups;
@@ -481,15 +483,27 @@ __device__ __forceinline__ void merge_round(const uint64_t* src, uint64_t* dst, 
 // keys).  Above: one run per block, then ceil(log8(runs)) merge rounds; 8 ways
 // because a key's searches are then bound by their round trips, not by their
 // instructions (a detect with 150,000 results: 234 us with 16 ways, 195 with 8).
+// publish (may be null): receives the finished status, and the working status
+// is zeroed for the next detect -- by one thread, once no block needs the
+// count any more (with at most kRun keys the other blocks return whether they
+// read the count or the zero).
 __global__ void __launch_bounds__(kSortThreads)
-k_sort_emit(uint64_t* keys, uint32_t cap, const DetectStatus* status, const double* est_table,
-            sp_candidate* out) {
+k_sort_emit(uint64_t* keys, uint32_t cap, DetectStatus* status, const double* est_table,
+            sp_candidate* out, DetectStatus* publish) {
   __shared__ uint64_t s_keys[kRun];
-  const uint32_t n = min(status->count, cap);        // the same for every block
-  if (n == 0) return;
+  const uint32_t n = min(status->count, cap);        // the same for every block (above kRun)
   const uint32_t tid = threadIdx.x;
+  auto hand_over = [&]() {
+    if (publish != nullptr && blockIdx.x == 0 && tid == 0) {
+      *publish = *status;
+      *status = DetectStatus{0u, 0u, 0ull};
+    }
+  };
   if (n <= kRun) {                                  // one block, in shared memory
     if (blockIdx.x != 0) return;
+    __syncthreads();                                // every thread of the block has the count
+    hand_over();
+    if (n == 0) return;
     uint32_t m = 2;
     while (m < n) m <<= 1;
     for (uint32_t i = tid; i < m; i += kSortThreads) s_keys[i] = i < n ? keys[i] : ~0ull;
@@ -518,6 +532,7 @@ k_sort_emit(uint64_t* keys, uint32_t cap, const DetectStatus* status, const doub
   // 2. merge rounds; the last one reads the key buffer and writes the records
   for (uint64_t w = kRun; w < n; w *= kWays) {
     grid.sync();
+    if (w == kRun) hand_over();                                    // every block has the count
     const uint64_t left = (n + w - 1) / w;                         // runs
     sp_candidate* to = left <= kWays ? out : nullptr;
     if (left <= 2) merge_round<2>(src, dst, to, est_table, n, w);
@@ -533,6 +548,31 @@ k_sort_emit(uint64_t* keys, uint32_t cap, const DetectStatus* status, const doub
 
 namespace {
 
+// Blocks of a kernel that a device holds at a given dynamic shared memory
+// size, asked once: the last answer is kept per kernel, packed into one word
+// (device + 1, shared memory, blocks), so that any thread may ask.
+template <typename Kernel>
+cudaError_t resident_blocks(Kernel kern, int threads, uint32_t smem, std::atomic<uint64_t>& last, int* blocks) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t key = ((uint64_t)(dev + 1) << 48) | ((uint64_t)smem << 24);
+  const uint64_t was = last.load(std::memory_order_acquire);
+  if ((was & ~0xFFFFFFull) == key) {
+    *blocks = (int)(was & 0xFFFFFFull);
+    return cudaSuccess;
+  }
+  int sms = 0, per_sm = 0;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem)) != cudaSuccess) return e;
+  *blocks = sms * per_sm;
+  last.store(key | (uint64_t)*blocks, std::memory_order_release);
+  return cudaSuccess;
+}
+
+// dynamic shared memory of k_detect for the largest SEA (4,096 bytes, unstaged) and the largest ring
+constexpr int kDetectSmemMost = kDetectWarps * (kHostQueue * 4 + 4096 * 2);
+
 template <bool kSliding, int kSeaRing>
 cudaError_t detect_launch_ring(const DevParams& d, const uint8_t* seav, const LdcaRead& ldca, const uint64_t* clock,
                                uint32_t k_slices, uint32_t z_theta, const Found& f, cudaStream_t s) {
@@ -540,16 +580,23 @@ cudaError_t detect_launch_ring(const DevParams& d, const uint8_t* seav, const Ld
                       (size_t)kDetectWarps * d.sea_bytes * sizeof(uint16_t) +
                       (size_t)kDetectWarps * kSeaRing * d.sea_bytes;
   auto kern = k_detect<kSliding, kSeaRing>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit is set to the same constant once per device: no call lowers it under another's launch
+  static std::atomic<uint64_t> limit_set{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kDetectThreads, smem);
-  if (per_sm < 1) per_sm = 1;
+  if (dev >= 64 || !((limit_set.load(std::memory_order_acquire) >> dev) & 1u)) {
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDetectSmemMost)) != cudaSuccess)
+      return e;
+    if (dev < 64) limit_set.fetch_or(1ull << dev, std::memory_order_release);
+  }
+  static std::atomic<uint64_t> resident{0};
+  int most = 0;
+  if ((e = resident_blocks(kern, kDetectThreads, (uint32_t)smem, resident, &most)) != cudaSuccess) return e;
+  if (most < 1) return cudaErrorInvalidConfiguration;
   const uint64_t n_sea = 1ull << d.r;
   uint64_t grid = (n_sea + kDetectWarps - 1) / kDetectWarps;
-  if (grid > (uint64_t)sms * per_sm) grid = (uint64_t)sms * per_sm;
+  if (grid > (uint64_t)most) grid = (uint64_t)most;
   kern<<<(unsigned)grid, kDetectThreads, smem, s>>>(d, seav, ldca, clock, k_slices, z_theta, f);
   return cudaGetLastError();
 }
@@ -584,20 +631,19 @@ cudaError_t launch_detect_sliding(const DevParams& d, const uint8_t* seav, const
   return detect_launch<true>(d, seav, a, clock, k, z_theta, keys, cap, max_join, status, s);
 }
 
-cudaError_t launch_sort_emit(uint64_t* keys, uint32_t cap, const DetectStatus* status,
+cudaError_t launch_sort_emit(uint64_t* keys, uint32_t cap, DetectStatus* status,
                              const double* est_table, uint32_t /*k_log2*/,
-                             sp_candidate* out, cudaStream_t s) {
+                             sp_candidate* out, DetectStatus* publish, cudaStream_t s) {
   // a cooperative grid (every block resident) of at most one block per SM,
   // and no more blocks than runs of the largest count
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sort_emit, kSortThreads, 0);
+  static std::atomic<uint64_t> resident{0};
+  int most = 0;
+  cudaError_t e = resident_blocks(k_sort_emit, kSortThreads, 0u, resident, &most);
   if (e != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  if (most < 1) return cudaErrorInvalidConfiguration;
   const uint32_t max_runs = (cap + kRun - 1) / kRun;
-  const unsigned grid = (unsigned)(max_runs < (uint32_t)sms ? (max_runs ? max_runs : 1u) : (uint32_t)sms);
-  void* args[] = {&keys, &cap, &status, &est_table, &out};
+  const unsigned grid = max_runs < (uint32_t)most ? (max_runs ? max_runs : 1u) : (unsigned)most;
+  void* args[] = {&keys, &cap, &status, &est_table, &out, &publish};
   e = cudaLaunchCooperativeKernel((const void*)k_sort_emit, dim3(grid), dim3(kSortThreads), args, 0, s);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();

@@ -207,8 +207,9 @@ cudaError_t launch_detect_sliding(const DevParams& d, const uint8_t* seav, const
                                   const uint8_t* st_ldca, const uint64_t* clock, uint32_t k, uint32_t z_theta,
                                   uint64_t* keys, uint32_t cap, uint64_t max_join, DetectStatus* status,
                                   cudaStream_t s);
-cudaError_t launch_sort_emit(uint64_t* keys, uint32_t cap, const DetectStatus* status,
+// publish (may be null): receives the status; *status is zeroed for the next detect then
+cudaError_t launch_sort_emit(uint64_t* keys, uint32_t cap, DetectStatus* status,
                              const double* est_table, uint32_t k_log2,
-                             sp_candidate* out, cudaStream_t s);
+                             sp_candidate* out, DetectStatus* publish, cudaStream_t s);
 
 }  // namespace sp

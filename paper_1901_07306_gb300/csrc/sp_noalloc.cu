@@ -138,7 +138,7 @@ extern "C" int sp_detect_noalloc(const sp_params* p, const uint8_t* dev_seav, co
   const uint64_t max_join = p->max_join ? p->max_join : (1ull << 26);
   if (sp::launch_detect(d, dev_seav, dev_ldca, zt, keys, cap, max_join, status, st) != cudaSuccess) return SP_ERR_CUDA;
   if (dev_out &&
-      sp::launch_sort_emit(keys, cap, status, est, p->k_log2, dev_out, st) != cudaSuccess) return SP_ERR_CUDA;
+      sp::launch_sort_emit(keys, cap, status, est, p->k_log2, dev_out, nullptr, st) != cudaSuccess) return SP_ERR_CUDA;
   // count and overflow flags to the caller's two words
   if (cudaMemcpyAsync(dev_status, status, 2 * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return SP_ERR_CUDA;

@@ -376,18 +376,24 @@ def sp_detect_async(ctx: int, router: int = 0, threshold: int = 0) -> int:
     return _check(lib.sp_detect_async(ctypes.c_void_p(ctx), router, threshold), "sp_detect_async")
 
 
+_FIRST_RECORDS = 2048            # records asked for before their number is known
+
+
 def sp_results(ctx: int, cap: int | None = None):
-    """Returns (records, n_total, status) for the last detect."""
+    """Returns (records, n_total, status) for the last detect; cap None: all."""
     n = ctypes.c_uint64()
-    if cap is None:
-        rc = lib.sp_results(ctypes.c_void_p(ctx), None, 0, ctypes.byref(n))
-        if rc not in (SP_OK, SP_ERR_TRUNCATED, SP_ERR_CANDIDATE_OVERFLOW):
-            _check(rc, "sp_results")
-        cap = n.value
-    out = np.zeros(max(cap, 1), CANDIDATE)
-    rc = lib.sp_results(ctypes.c_void_p(ctx), ctypes.c_void_p(out.ctypes.data), cap, ctypes.byref(n))
-    _check(rc, "sp_results", ok=(SP_OK, SP_ERR_TRUNCATED, SP_ERR_CANDIDATE_OVERFLOW))
-    written = min(cap, n.value, sp_get_params(ctx).max_candidates)
+    ok = (SP_OK, SP_ERR_TRUNCATED, SP_ERR_CANDIDATE_OVERFLOW)
+    ask = _FIRST_RECORDS if cap is None else cap
+    while True:
+        out = (np.empty if cap is None else np.zeros)(max(ask, 1), CANDIDATE)
+        rc = lib.sp_results(ctypes.c_void_p(ctx), ctypes.c_void_p(out.ctypes.data), ask, ctypes.byref(n))
+        _check(rc, "sp_results", ok=ok)
+        if cap is not None or n.value <= ask:
+            break
+        cap = ask = n.value                          # one more call with room for all
+    written = min(ask, n.value)
+    if rc == SP_ERR_CANDIDATE_OVERFLOW:
+        written = min(written, sp_get_params(ctx).max_candidates)
     return out[:written], n.value, rc
 
 
