@@ -1,6 +1,6 @@
 // sp_detect.cu -- end-of-window restore and filter (Sec. 3.2-3.3, Sec. 4.2).
 //
-// k_detect: one warp per SEA (grid-stride over the 2^r SEAs).
+// k_detect: one warp per SEA (a block's warps share its part of the 2^r SEAs).
 //   1. HSE(i): lanes test the SEs of a row for weight >= 3 (4 per lane per
 //      32-bit load on rows of 128+ SEs) and a ballot/popc prefix compacts the
 //      hot columns into a per-warp list in shared memory (Sec. 3.2, "hot SE").
@@ -47,12 +47,11 @@ constexpr int kDetectWarps = 8;
 constexpr int kDetectThreads = kDetectWarps * 32;
 constexpr int kHostQueue = 256;                  // complete tuples queued per warp
 constexpr uint32_t kFull = 0xFFFFFFFFu;
+constexpr uint32_t kTestAt = 32;                  // queued hosts a warp tests together (fewer at its end)
 constexpr int kPending = 64;                     // found keys a warp holds back before it appends them
-// SEAs of a multiple of 16 bytes, up to 1 KiB, are staged in shared memory: a
-// ring of 4 SEAs per warp (3 above 512 bytes, so that four blocks still share
-// an SM), filled one SEA less than the ring ahead of use
+// SEAs of a multiple of 16 bytes, up to 1 KiB, are staged in shared memory:
+// two per warp, the next one copied while the current one is worked on
 constexpr uint32_t kStagedSea = 1024;
-constexpr int sea_ring(uint32_t sea_bytes) { return sea_bytes <= 512 ? 4 : 3; }
 
 // 16-byte asynchronous copy from global to shared memory (one per lane)
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
@@ -238,17 +237,22 @@ __device__ void test_queue(const DevParams& d, const LdcaRead& ldca, const uint3
   }
 }
 
-template <bool kSliding, int kSeaRing>             // kSeaRing: SEAs per warp staged in shared memory, 0 = none
+// A warp's time goes to latencies (a core-link SEA has 1.4 hot SEs per row and
+// one or two hosts to test): its SEA's copy, the join's dependent reads, one
+// round trip to the LDC lines per test pass.  The next SEA is copied
+// meanwhile; hosts are tested two a pass once kTestAt are queued or the warp
+// is done, not one or two after every SEA; and the warps of a block take its
+// SEAs from one counter, since SEAs differ.  DETFIG
+template <bool kSliding, bool kStaged>
 __global__ void __launch_bounds__(kDetectThreads, 4)
 k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uint64_t* __restrict__ clock,
          uint32_t k_slices, uint32_t z_theta, Found f) {
-  constexpr bool staged = kSeaRing > 0;
   extern __shared__ __align__(16) uint32_t s_dyn[];
   if (kSliding) {                                   // the window of the router's current slice
     ldca.cur4 = ((uint32_t)(*clock % 255u) + 1u) * 0x01010101u;
     ldca.k4 = k_slices * 0x01010101u;
   }
-  __shared__ uint32_t s_queue_n[kDetectWarps];
+  __shared__ uint32_t s_queue_n[kDetectWarps], s_next;
   __shared__ uint64_t s_pending[kDetectWarps][kPending];
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   uint32_t* queue = s_dyn + warp * kHostQueue;           // [kDetectWarps][kHostQueue] IPs
@@ -256,43 +260,50 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
   uint16_t* lists = reinterpret_cast<uint16_t*>(s_dyn + kDetectWarps * kHostQueue) + warp * d.sea_bytes;
   Pending pend{s_pending[warp], 0u};
   if (lane == 0) *queue_n = 0;
-  __syncwarp();
+  if (threadIdx.x == 0) s_next = 0;
+  __syncthreads();
   const uint32_t n_sea = 1u << d.r;
-  const uint32_t stride = gridDim.x * kDetectWarps;
-  // staged SEAs (16-byte aligned SEAV and SEA size): the warp's ring of
-  // kSeaRing SEAs after the lists; 16 bytes per lane and copy by cp.async,
-  // one commit group per SEA (empty past the last SEA, so that the count of
-  // groups in flight stays fixed)
-  uint8_t* ring = reinterpret_cast<uint8_t*>(s_dyn + kDetectWarps * kHostQueue) +
-                  (size_t)kDetectWarps * d.sea_bytes * sizeof(uint16_t) + (size_t)warp * kSeaRing * d.sea_bytes;
+  // the block's SEAs are blockIdx.x, blockIdx.x + gridDim.x, ...; a warp takes the next one
+  auto next_sea = [&]() {
+    uint32_t k = 0;
+    if (lane == 0) k = atomicAdd(&s_next, 1u);
+    k = __shfl_sync(kFull, k, 0);
+    const uint64_t rp = (uint64_t)blockIdx.x + (uint64_t)k * gridDim.x;
+    return rp < n_sea ? (uint32_t)rp : n_sea;
+  };
+  // staged SEAs (16-byte aligned SEAV and SEA size): the warp's two buffers
+  // after the lists; 16 bytes per lane and copy by cp.async, one commit group
+  // per SEA (empty past the last SEA, so that the count of groups in flight
+  // stays fixed)
+  uint8_t* buffers = reinterpret_cast<uint8_t*>(s_dyn + kDetectWarps * kHostQueue) +
+                     (size_t)kDetectWarps * d.sea_bytes * sizeof(uint16_t) + (size_t)warp * 2u * d.sea_bytes;
   auto stage_sea = [&](uint32_t rp, uint32_t slot) {
     if (rp < n_sea)
       for (uint32_t o = 16u * lane; o < d.sea_bytes; o += 512u)
-        cp_async16(ring + slot * d.sea_bytes + o, seav + (uint64_t)rp * d.sea_bytes + o);
+        cp_async16(buffers + slot * d.sea_bytes + o, seav + (uint64_t)rp * d.sea_bytes + o);
     cp_async_commit();
   };
-  uint32_t rp = blockIdx.x * kDetectWarps + warp;
-  if (staged) {
-#pragma unroll
-    for (int j = 0; j < kSeaRing - 1; ++j) stage_sea(rp + (uint32_t)j * stride, (uint32_t)j);
-  }
+  uint32_t rp = next_sea(), slot = 0;
+  if (kStaged) stage_sea(rp, 0u);
   uint32_t join_local = 0;
   bool stop = false;
-  for (uint32_t it = 0; rp < n_sea && !stop; rp += stride, ++it) {
+  while (rp < n_sea && !stop) {
     // the join-bound flag (warp-uniform: lane 0 reads it, every lane sees its
     // value) is read here and tested after this SEA, so the read overlaps the
     // work; a warp stops at most one SEA later than the bound was hit
     const uint32_t ov = lane == 0 ? *reinterpret_cast<volatile uint32_t*>(&f.status->overflow) : 0u;
     const uint8_t* sea = seav + (uint64_t)rp * d.sea_bytes;
-    if (staged) {
-      // the SEA kSeaRing - 1 ahead goes to the slot this warp read last
-      // (every lane passed the __syncwarp at the end of that iteration); then
-      // wait for this SEA's copy and make every lane's bytes visible
-      constexpr uint32_t R = staged ? kSeaRing : 1;
-      stage_sea(rp + (R - 1) * stride, (it + R - 1) % R);
-      cp_async_wait<R - 1>();
+    uint32_t rp_next = n_sea;
+    if (kStaged) {
+      // the next SEA goes to the buffer this warp read last (every lane passed
+      // the __syncwarp at the end of that turn); then wait for this SEA's copy
+      // and make every lane's bytes visible
+      rp_next = next_sea();
+      stage_sea(rp_next, slot ^ 1u);
+      cp_async_wait<1>();
       __syncwarp();
-      sea = ring + (it % R) * d.sea_bytes;
+      sea = buffers + slot * d.sea_bytes;
+      slot ^= 1u;
     }
     // 1. hot SEs per row
     uint32_t cnt[8];
@@ -334,15 +345,21 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
     if (!empty) {
       // 2. lanes split HSE(0) x HSE(1); depth-first over the remaining rows
       const uint32_t n1 = d.sr > 1 ? cnt[1] : 1u;
-      const uint32_t total = cnt[0] * n1;
+      const uint32_t total = cnt[0] * n1;                       // <= 2^24: exact as a float
+      const float inv1 = 1.0f / (float)n1;
       for (uint32_t t = lane; t < total && !stop; t += 32) {
-        const uint32_t c0 = lists[d.row_off[0] + t / n1];
+        // t / n1 and t mod n1: a float quotient is off by one at most
+        uint32_t t0 = (uint32_t)((float)t * inv1);
+        int t1 = (int)(t - t0 * n1);
+        if (t1 < 0) { --t0; t1 += (int)n1; }
+        if (t1 >= (int)n1) { ++t0; t1 -= (int)n1; }
+        const uint32_t c0 = lists[d.row_off[0] + t0];
         uint32_t km = d.cover[0];
         uint32_t kv = spread_idx(c0, d.isb[0], d.L);
         uint32_t seu = sea[d.row_off[0] + c0];
         uint32_t start = 1;
         if (d.sr > 1) {
-          const uint32_t c1 = lists[d.row_off[1] + t % n1];
+          const uint32_t c1 = lists[d.row_off[1] + (uint32_t)t1];
           const uint32_t v1 = spread_idx(c1, d.isb[1], d.L);
           if (((v1 ^ kv) & d.cover[1] & km) != 0u) continue;
           seu &= sea[d.row_off[1] + c1];
@@ -382,17 +399,21 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
       }
     }
     __syncwarp();
-    // 3. the warp's LDCA test of this SEA's complete tuples
-    const uint32_t nq = min(*queue_n, (uint32_t)kHostQueue);
-    if (nq) test_queue<kSliding>(d, ldca, queue, nq, z_theta, f, pend, lane);
-    __syncwarp();
-    if (lane == 0) *queue_n = 0;
+    // 3. the warp's LDCA test of the queued complete tuples
+    const uint32_t nq = *queue_n;
+    if (nq >= kTestAt) {
+      test_queue<kSliding>(d, ldca, queue, min(nq, (uint32_t)kHostQueue), z_theta, f, pend, lane);
+      __syncwarp();
+      if (lane == 0) *queue_n = 0;
+    }
     __syncwarp();
     const bool bound = (__shfl_sync(kFull, ov, 0) & 2u) != 0u;
     stop = __any_sync(kFull, stop) || bound;
+    rp = kStaged ? rp_next : next_sea();
   }
+  if (*queue_n != 0u) test_queue<kSliding>(d, ldca, queue, min(*queue_n, (uint32_t)kHostQueue), z_theta, f, pend, lane);
   flush_pending(pend, f, lane);
-  if (staged) cp_async_wait<0>();                  // no copy in flight at exit
+  if (kStaged) cp_async_wait<0>();                 // no copy in flight at exit
   join_local = __reduce_add_sync(kFull, join_local);           // one atomic per warp
   if (lane == 0 && join_local) atomicAdd(reinterpret_cast<unsigned long long*>(&f.status->join), (unsigned long long)join_local);
 }
@@ -570,16 +591,16 @@ cudaError_t resident_blocks(Kernel kern, int threads, uint32_t smem, std::atomic
   return cudaSuccess;
 }
 
-// dynamic shared memory of k_detect for the largest SEA (4,096 bytes, unstaged) and the largest ring
+// dynamic shared memory of k_detect for the largest SEA (4,096 bytes, unstaged); staged ones need less
 constexpr int kDetectSmemMost = kDetectWarps * (kHostQueue * 4 + 4096 * 2);
 
-template <bool kSliding, int kSeaRing>
-cudaError_t detect_launch_ring(const DevParams& d, const uint8_t* seav, const LdcaRead& ldca, const uint64_t* clock,
-                               uint32_t k_slices, uint32_t z_theta, const Found& f, cudaStream_t s) {
+template <bool kSliding, bool kStaged>
+cudaError_t detect_launch_staged(const DevParams& d, const uint8_t* seav, const LdcaRead& ldca, const uint64_t* clock,
+                                 uint32_t k_slices, uint32_t z_theta, const Found& f, cudaStream_t s) {
   const size_t smem = (size_t)kDetectWarps * kHostQueue * sizeof(uint32_t) +
                       (size_t)kDetectWarps * d.sea_bytes * sizeof(uint16_t) +
-                      (size_t)kDetectWarps * kSeaRing * d.sea_bytes;
-  auto kern = k_detect<kSliding, kSeaRing>;
+                      (kStaged ? (size_t)kDetectWarps * 2u * d.sea_bytes : 0u);
+  auto kern = k_detect<kSliding, kStaged>;
   // the limit is set to the same constant once per device: no call lowers it under another's launch
   static std::atomic<uint64_t> limit_set{0};
   int dev = 0;
@@ -606,12 +627,10 @@ cudaError_t detect_launch(const DevParams& d, const uint8_t* seav, const LdcaRea
                           uint32_t k_slices, uint32_t z_theta, uint64_t* keys, uint32_t cap, uint64_t max_join,
                           DetectStatus* status, cudaStream_t s) {
   const Found f{keys, cap, max_join, status};
-  // staged SEAs need 16-byte copies; above kStagedSea a ring would cost blocks
+  // staged SEAs need 16-byte copies; above kStagedSea the buffers would cost blocks
   if ((d.sea_bytes & 15u) != 0u || d.sea_bytes > kStagedSea || ((uintptr_t)seav & 15u) != 0u)
-    return detect_launch_ring<kSliding, 0>(d, seav, ldca, clock, k_slices, z_theta, f, s);
-  if (sea_ring(d.sea_bytes) == 4)
-    return detect_launch_ring<kSliding, 4>(d, seav, ldca, clock, k_slices, z_theta, f, s);
-  return detect_launch_ring<kSliding, 3>(d, seav, ldca, clock, k_slices, z_theta, f, s);
+    return detect_launch_staged<kSliding, false>(d, seav, ldca, clock, k_slices, z_theta, f, s);
+  return detect_launch_staged<kSliding, true>(d, seav, ldca, clock, k_slices, z_theta, f, s);
 }
 
 }  // namespace
