@@ -62,6 +62,12 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
 
+// How k_detect reads an SEA: rows from global memory, rows of a staged SEA, or
+// a staged SEA of four rows of 128 SEs whose LP has at most 24 bits (profiles D,
+// D3, S and K12).
+enum class Form { kDirect, kStaged, kFour };
+__host__ __device__ constexpr uint32_t list_bytes(Form form) { return form == Form::kFour ? 4u : 2u; }   // per SE
+
 struct Found {
   uint64_t* keys;
   uint32_t cap;
@@ -243,10 +249,11 @@ __device__ void test_queue(const DevParams& d, const LdcaRead& ldca, const uint3
 // meanwhile; hosts are tested two a pass once kTestAt are queued or the warp
 // is done, not one or two after every SEA; and the warps of a block take its
 // SEAs from one counter, since SEAs differ.  DETFIG
-template <bool kSliding, bool kStaged>
+template <bool kSliding, Form kForm>
 __global__ void __launch_bounds__(kDetectThreads, 4)
 k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uint64_t* __restrict__ clock,
          uint32_t k_slices, uint32_t z_theta, Found f) {
+  constexpr bool kStaged = kForm != Form::kDirect;
   extern __shared__ __align__(16) uint32_t s_dyn[];
   if (kSliding) {                                   // the window of the router's current slice
     ldca.cur4 = ((uint32_t)(*clock % 255u) + 1u) * 0x01010101u;
@@ -257,7 +264,9 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   uint32_t* queue = s_dyn + warp * kHostQueue;           // [kDetectWarps][kHostQueue] IPs
   uint32_t* queue_n = &s_queue_n[warp];
+  // the warp's hot SEs, row by row: columns (uint16), with kFour whole entries (uint32)
   uint16_t* lists = reinterpret_cast<uint16_t*>(s_dyn + kDetectWarps * kHostQueue) + warp * d.sea_bytes;
+  uint32_t* entries = s_dyn + kDetectWarps * kHostQueue + warp * 512u;
   Pending pend{s_pending[warp], 0u};
   if (lane == 0) *queue_n = 0;
   if (threadIdx.x == 0) s_next = 0;
@@ -276,13 +285,18 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
   // per SEA (empty past the last SEA, so that the count of groups in flight
   // stays fixed)
   uint8_t* buffers = reinterpret_cast<uint8_t*>(s_dyn + kDetectWarps * kHostQueue) +
-                     (size_t)kDetectWarps * d.sea_bytes * sizeof(uint16_t) + (size_t)warp * 2u * d.sea_bytes;
+                     (size_t)kDetectWarps * d.sea_bytes * list_bytes(kForm) + (size_t)warp * 2u * d.sea_bytes;
   auto stage_sea = [&](uint32_t rp, uint32_t slot) {
     if (rp < n_sea)
       for (uint32_t o = 16u * lane; o < d.sea_bytes; o += 512u)
         cp_async16(buffers + slot * d.sea_bytes + o, seav + (uint64_t)rp * d.sea_bytes + o);
     cp_async_commit();
   };
+  // kFour: this lane's 16 SEs of an SEA are in row lane / 8; LP bits that row i
+  // shares with the rows before it
+  const uint32_t my_isb = kForm == Form::kFour ? d.isb[lane >> 3] : 0u;
+  const uint32_t shared1 = d.cover[1] & d.cover[0], shared2 = d.cover[2] & (d.cover[0] | d.cover[1]);
+  const uint32_t shared3 = d.cover[3] & (d.cover[0] | d.cover[1] | d.cover[2]);
   uint32_t rp = next_sea(), slot = 0;
   if (kStaged) stage_sea(rp, 0u);
   uint32_t join_local = 0;
@@ -305,95 +319,152 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
       sea = buffers + slot * d.sea_bytes;
       slot ^= 1u;
     }
-    // 1. hot SEs per row
-    uint32_t cnt[8];
-    bool empty = false;
-    for (uint32_t i = 0; i < d.sr; ++i) {
-      const uint32_t sc = 1u << d.ibn[i];
-      const uint8_t* row = sea + d.row_off[i];
-      uint32_t n = 0;
-      if (sc >= 128 && ((uintptr_t)row & 3u) == 0) {
-        // rows of 128+ SEs, word aligned: 4 SEs per lane per load; the list
-        // is ordered by (byte of the word, lane), which only changes the order
-        // in which candidates are tried
-        for (uint32_t c0 = 0; c0 < sc; c0 += 128) {
-          const uint32_t w = *reinterpret_cast<const uint32_t*>(row + c0 + 4 * lane);
+    if (kForm == Form::kFour) {
+      // 1. hot SEs: a lane looks at 16 SEs at once (weights side by side in a
+      // word), a scan over the row's 8 lanes gives the places; an entry is the
+      // column's LP bits (Eq. 3) with the SE above them
+      const uint4 x = *reinterpret_cast<const uint4*>(sea + 16u * lane);
+      const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+      uint32_t hot = 0;
 #pragma unroll
-          for (uint32_t j = 0; j < 4; ++j) {
-            const bool hot = __popc((w >> (8 * j)) & 0xFFu) >= 3;
+      for (int j = 0; j < 4; ++j) {
+        uint32_t y = w[j] - ((w[j] >> 1) & 0x55555555u);
+        y = (y & 0x33333333u) + ((y >> 2) & 0x33333333u);
+        y = (y + (y >> 4)) & 0x0F0F0F0Fu;
+        y = ((y + 0x7D7D7D7Du) >> 7) & 0x01010101u;                // weight >= 3, a bit per byte
+        hot |= (((y * 0x00204081u) >> 21) & 0xFu) << (4 * j);
+      }
+      uint32_t at = __popc(hot);
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, at, o, 8);
+        if ((lane & 7u) >= (uint32_t)o) at += y;
+      }
+      const uint32_t row_n = __shfl_sync(kFull, at, 7, 8);
+      if (!__any_sync(kFull, row_n == 0u)) {                       // a row without a hot SE: no tuple
+        at -= __popc(hot);
+        while (hot != 0u) {
+          const uint32_t j = __ffs(hot) - 1u;
+          hot &= hot - 1u;
+          entries[(lane & 24u) * 16u + at++] =
+              spread_idx(16u * (lane & 7u) + j, my_isb, d.L) | (uint32_t)sea[16u * lane + j] << 24;
+        }
+        const uint32_t n0 = __shfl_sync(kFull, row_n, 0), n1 = __shfl_sync(kFull, row_n, 8);
+        const uint32_t n2 = __shfl_sync(kFull, row_n, 16), n3 = __shfl_sync(kFull, row_n, 24);
+        __syncwarp();
+        // 2. lanes split HSE(0) x HSE(1); a partial tuple is its LP bits with its
+        // SEU above them, dropped as soon as shared bits differ or the SEU is light
+        constexpr uint32_t kLp = 0x00FFFFFFu;
+        const uint32_t total = n0 * n1;
+        for (uint32_t t = lane; t < total && !stop; t += 32) {
+          const uint32_t t0 = t / n1;
+          const uint32_t e0 = entries[t0], e1 = entries[128u + t - t0 * n1];
+          if (((e0 ^ e1) & shared1) != 0u) continue;
+          const uint32_t p = ((e0 | e1) & kLp) | (e0 & e1 & ~kLp);
+          if (__popc(p >> 24) < 3) continue;
+          for (uint32_t i = 0; i < n2 && !stop; ++i) {
+            const uint32_t e2 = entries[256u + i];
+            const uint32_t q = ((p | e2) & kLp) | (p & e2 & ~kLp);
+            if (((p ^ e2) & shared2) != 0u || __popc(q >> 24) < 3) continue;
+            for (uint32_t k = 0; k < n3 && !stop; ++k) {
+              const uint32_t e3 = entries[384u + k];
+              if (((q ^ e3) & shared3) != 0u || __popc((q & e3) >> 24) < 3) continue;
+              if (!emit_lp<kSliding>(d, ldca, rp, (q | e3) & kLp, z_theta, f, join_local, queue, queue_n)) stop = true;
+            }
+          }
+        }
+      }
+    } else {
+      // 1. hot SEs per row
+      uint32_t cnt[8];
+      bool empty = false;
+      for (uint32_t i = 0; i < d.sr; ++i) {
+        const uint32_t sc = 1u << d.ibn[i];
+        const uint8_t* row = sea + d.row_off[i];
+        uint32_t n = 0;
+        if (sc >= 128 && ((uintptr_t)row & 3u) == 0) {
+          // rows of 128+ SEs, word aligned: 4 SEs per lane per load; the list
+          // is ordered by (byte of the word, lane), which only changes the order
+          // in which candidates are tried
+          for (uint32_t c0 = 0; c0 < sc; c0 += 128) {
+            const uint32_t w = *reinterpret_cast<const uint32_t*>(row + c0 + 4 * lane);
+  #pragma unroll
+            for (uint32_t j = 0; j < 4; ++j) {
+              const bool hot = __popc((w >> (8 * j)) & 0xFFu) >= 3;
+              const uint32_t bal = __ballot_sync(kFull, hot);
+              if (hot) lists[d.row_off[i] + n + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(c0 + 4 * lane + j);
+              n += __popc(bal);
+            }
+          }
+        } else {
+          for (uint32_t c0 = 0; c0 < sc; c0 += 32) {
+            const uint32_t c = c0 + lane;
+            const bool hot = c < sc && __popc((uint32_t)row[c]) >= 3;
             const uint32_t bal = __ballot_sync(kFull, hot);
-            if (hot) lists[d.row_off[i] + n + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(c0 + 4 * lane + j);
+            if (hot) lists[d.row_off[i] + n + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)c;
             n += __popc(bal);
           }
         }
-      } else {
-        for (uint32_t c0 = 0; c0 < sc; c0 += 32) {
-          const uint32_t c = c0 + lane;
-          const bool hot = c < sc && __popc((uint32_t)row[c]) >= 3;
-          const uint32_t bal = __ballot_sync(kFull, hot);
-          if (hot) lists[d.row_off[i] + n + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)c;
-          n += __popc(bal);
+        cnt[i] = n;
+        if (n == 0) {                                  // no tuple can cover this row: the SEA yields nothing
+          empty = true;
+          break;
         }
       }
-      cnt[i] = n;
-      if (n == 0) {                                  // no tuple can cover this row: the SEA yields nothing
-        empty = true;
-        break;
-      }
-    }
-    __syncwarp();
-    if (!empty) {
-      // 2. lanes split HSE(0) x HSE(1); depth-first over the remaining rows
-      const uint32_t n1 = d.sr > 1 ? cnt[1] : 1u;
-      const uint32_t total = cnt[0] * n1;                       // <= 2^24: exact as a float
-      const float inv1 = 1.0f / (float)n1;
-      for (uint32_t t = lane; t < total && !stop; t += 32) {
-        // t / n1 and t mod n1: a float quotient is off by one at most
-        uint32_t t0 = (uint32_t)((float)t * inv1);
-        int t1 = (int)(t - t0 * n1);
-        if (t1 < 0) { --t0; t1 += (int)n1; }
-        if (t1 >= (int)n1) { ++t0; t1 -= (int)n1; }
-        const uint32_t c0 = lists[d.row_off[0] + t0];
-        uint32_t km = d.cover[0];
-        uint32_t kv = spread_idx(c0, d.isb[0], d.L);
-        uint32_t seu = sea[d.row_off[0] + c0];
-        uint32_t start = 1;
-        if (d.sr > 1) {
-          const uint32_t c1 = lists[d.row_off[1] + (uint32_t)t1];
-          const uint32_t v1 = spread_idx(c1, d.isb[1], d.L);
-          if (((v1 ^ kv) & d.cover[1] & km) != 0u) continue;
-          seu &= sea[d.row_off[1] + c1];
-          if (__popc(seu) < 3) continue;
-          km |= d.cover[1];
-          kv |= v1;
-          start = 2;
-        }
-        if (start == d.sr) {
-          if (!emit_lp<kSliding>(d, ldca, rp, kv, z_theta, f, join_local, queue, queue_n)) stop = true;
-          continue;
-        }
-        uint32_t pos[8], skm[8], skv[8], sseu[8];
-        int dd = (int)start;
-        pos[dd] = 0; skm[dd] = km; skv[dd] = kv; sseu[dd] = seu;
-        while (dd >= (int)start && !stop) {
-          if (pos[dd] >= cnt[dd]) {
-            if (--dd >= (int)start) ++pos[dd];
+      __syncwarp();
+      if (!empty) {
+        // 2. lanes split HSE(0) x HSE(1); depth-first over the remaining rows
+        const uint32_t n1 = d.sr > 1 ? cnt[1] : 1u;
+        const uint32_t total = cnt[0] * n1;                       // <= 2^24: exact as a float
+        const float inv1 = 1.0f / (float)n1;
+        for (uint32_t t = lane; t < total && !stop; t += 32) {
+          // t / n1 and t mod n1: a float quotient is off by one at most
+          uint32_t t0 = (uint32_t)((float)t * inv1);
+          int t1 = (int)(t - t0 * n1);
+          if (t1 < 0) { --t0; t1 += (int)n1; }
+          if (t1 >= (int)n1) { ++t0; t1 -= (int)n1; }
+          const uint32_t c0 = lists[d.row_off[0] + t0];
+          uint32_t km = d.cover[0];
+          uint32_t kv = spread_idx(c0, d.isb[0], d.L);
+          uint32_t seu = sea[d.row_off[0] + c0];
+          uint32_t start = 1;
+          if (d.sr > 1) {
+            const uint32_t c1 = lists[d.row_off[1] + (uint32_t)t1];
+            const uint32_t v1 = spread_idx(c1, d.isb[1], d.L);
+            if (((v1 ^ kv) & d.cover[1] & km) != 0u) continue;
+            seu &= sea[d.row_off[1] + c1];
+            if (__popc(seu) < 3) continue;
+            km |= d.cover[1];
+            kv |= v1;
+            start = 2;
+          }
+          if (start == d.sr) {
+            if (!emit_lp<kSliding>(d, ldca, rp, kv, z_theta, f, join_local, queue, queue_n)) stop = true;
             continue;
           }
-          const uint32_t c = lists[d.row_off[dd] + pos[dd]];
-          const uint32_t v = spread_idx(c, d.isb[dd], d.L);
-          const uint32_t s2 = sseu[dd] & sea[d.row_off[dd] + c];
-          if (((v ^ skv[dd]) & d.cover[dd] & skm[dd]) == 0u && __popc(s2) >= 3) {
-            if (dd == (int)d.sr - 1) {
-              if (!emit_lp<kSliding>(d, ldca, rp, skv[dd] | v, z_theta, f, join_local, queue, queue_n)) stop = true;
-              ++pos[dd];
-            } else {
-              const int nx = dd + 1;
-              pos[nx] = 0; skm[nx] = skm[dd] | d.cover[dd]; skv[nx] = skv[dd] | v; sseu[nx] = s2;
-              dd = nx;
+          uint32_t pos[8], skm[8], skv[8], sseu[8];
+          int dd = (int)start;
+          pos[dd] = 0; skm[dd] = km; skv[dd] = kv; sseu[dd] = seu;
+          while (dd >= (int)start && !stop) {
+            if (pos[dd] >= cnt[dd]) {
+              if (--dd >= (int)start) ++pos[dd];
+              continue;
             }
-          } else {
-            ++pos[dd];
+            const uint32_t c = lists[d.row_off[dd] + pos[dd]];
+            const uint32_t v = spread_idx(c, d.isb[dd], d.L);
+            const uint32_t s2 = sseu[dd] & sea[d.row_off[dd] + c];
+            if (((v ^ skv[dd]) & d.cover[dd] & skm[dd]) == 0u && __popc(s2) >= 3) {
+              if (dd == (int)d.sr - 1) {
+                if (!emit_lp<kSliding>(d, ldca, rp, skv[dd] | v, z_theta, f, join_local, queue, queue_n)) stop = true;
+                ++pos[dd];
+              } else {
+                const int nx = dd + 1;
+                pos[nx] = 0; skm[nx] = skm[dd] | d.cover[dd]; skv[nx] = skv[dd] | v; sseu[nx] = s2;
+                dd = nx;
+              }
+            } else {
+              ++pos[dd];
+            }
           }
         }
       }
@@ -594,13 +665,13 @@ cudaError_t resident_blocks(Kernel kern, int threads, uint32_t smem, std::atomic
 // dynamic shared memory of k_detect for the largest SEA (4,096 bytes, unstaged); staged ones need less
 constexpr int kDetectSmemMost = kDetectWarps * (kHostQueue * 4 + 4096 * 2);
 
-template <bool kSliding, bool kStaged>
-cudaError_t detect_launch_staged(const DevParams& d, const uint8_t* seav, const LdcaRead& ldca, const uint64_t* clock,
+template <bool kSliding, Form kForm>
+cudaError_t detect_launch_form(const DevParams& d, const uint8_t* seav, const LdcaRead& ldca, const uint64_t* clock,
                                  uint32_t k_slices, uint32_t z_theta, const Found& f, cudaStream_t s) {
   const size_t smem = (size_t)kDetectWarps * kHostQueue * sizeof(uint32_t) +
-                      (size_t)kDetectWarps * d.sea_bytes * sizeof(uint16_t) +
-                      (kStaged ? (size_t)kDetectWarps * 2u * d.sea_bytes : 0u);
-  auto kern = k_detect<kSliding, kStaged>;
+                      (size_t)kDetectWarps * d.sea_bytes * list_bytes(kForm) +
+                      (kForm != Form::kDirect ? (size_t)kDetectWarps * 2u * d.sea_bytes : 0u);
+  auto kern = k_detect<kSliding, kForm>;
   // the limit is set to the same constant once per device: no call lowers it under another's launch
   static std::atomic<uint64_t> limit_set{0};
   int dev = 0;
@@ -629,8 +700,10 @@ cudaError_t detect_launch(const DevParams& d, const uint8_t* seav, const LdcaRea
   const Found f{keys, cap, max_join, status};
   // staged SEAs need 16-byte copies; above kStagedSea the buffers would cost blocks
   if ((d.sea_bytes & 15u) != 0u || d.sea_bytes > kStagedSea || ((uintptr_t)seav & 15u) != 0u)
-    return detect_launch_staged<kSliding, false>(d, seav, ldca, clock, k_slices, z_theta, f, s);
-  return detect_launch_staged<kSliding, true>(d, seav, ldca, clock, k_slices, z_theta, f, s);
+    return detect_launch_form<kSliding, Form::kDirect>(d, seav, ldca, clock, k_slices, z_theta, f, s);
+  const bool four = d.sr == 4 && d.L <= 24 && d.ibn[0] == 7 && d.ibn[1] == 7 && d.ibn[2] == 7 && d.ibn[3] == 7;
+  return four ? detect_launch_form<kSliding, Form::kFour>(d, seav, ldca, clock, k_slices, z_theta, f, s)
+              : detect_launch_form<kSliding, Form::kStaged>(d, seav, ldca, clock, k_slices, z_theta, f, s);
 }
 
 }  // namespace
