@@ -99,36 +99,18 @@ __device__ __forceinline__ uint64_t ldc_line(const DevParams& d, uint32_t ip, ui
   return (uint64_t)((i << d.lc_log2) | col) << (d.k_log2 - 5u);
 }
 
+// z0 of one host in one lane: the rare fallback of a full queue, kept small
+// (it is inlined into the join, whose registers count)
 template <bool kSliding>
 __device__ __forceinline__ uint32_t ldc_zeros(const DevParams& d, const LdcaRead& a, uint32_t ip) {
   const uint32_t wpl = 1u << (d.k_log2 - 5u);
-  uint64_t line[8];
-  for (uint32_t i = 0; i < d.lr; ++i) line[i] = ldc_line(d, ip, i);
   uint32_t ones = 0;
-  if (kSliding) {
-    for (uint32_t w = 0; w < wpl; ++w) {
-      uint32_t u = ldc_word<true>(a, line[0] + w);
-      for (uint32_t i = 1; i < d.lr; ++i) u &= ldc_word<true>(a, line[i] + w);
-      ones += __popc(u);
-    }
-    return (1u << d.k_log2) - ones;
-  }
-  const uint32_t* ldca = a.bits;
-  if (wpl >= 4) {
-    for (uint32_t w = 0; w < wpl; w += 4) {
-      uint4 u = *reinterpret_cast<const uint4*>(ldca + line[0] + w);
-      for (uint32_t i = 1; i < d.lr; ++i) {
-        const uint4 v = *reinterpret_cast<const uint4*>(ldca + line[i] + w);
-        u.x &= v.x; u.y &= v.y; u.z &= v.z; u.w &= v.w;
-      }
-      ones += __popc(u.x) + __popc(u.y) + __popc(u.z) + __popc(u.w);
-    }
-  } else {
-    for (uint32_t w = 0; w < wpl; ++w) {
-      uint32_t u = ldca[line[0] + w];
-      for (uint32_t i = 1; i < d.lr; ++i) u &= ldca[line[i] + w];
-      ones += __popc(u);
-    }
+#pragma unroll 1
+  for (uint32_t w = 0; w < wpl; ++w) {
+    uint32_t u = kFull;
+#pragma unroll 1
+    for (uint32_t i = 0; i < d.lr; ++i) u &= ldc_word<kSliding>(a, ldc_line(d, ip, i) + w);
+    ones += __popc(u);
   }
   return (1u << d.k_log2) - ones;
 }
@@ -250,7 +232,7 @@ __device__ void test_queue(const DevParams& d, const LdcaRead& ldca, const uint3
 // is done, not one or two after every SEA; and the warps of a block take its
 // SEAs from one counter, since SEAs differ.  DETFIG
 template <bool kSliding, Form kForm>
-__global__ void __launch_bounds__(kDetectThreads, 4)
+__global__ void __launch_bounds__(kDetectThreads, kForm == Form::kFour ? 5 : 4)
 k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uint64_t* __restrict__ clock,
          uint32_t k_slices, uint32_t z_theta, Found f) {
   constexpr bool kStaged = kForm != Form::kDirect;
