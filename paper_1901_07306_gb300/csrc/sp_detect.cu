@@ -337,9 +337,10 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
         // 2. lanes split HSE(0) x HSE(1); a partial tuple is its LP bits with its
         // SEU above them, dropped as soon as shared bits differ or the SEU is light
         constexpr uint32_t kLp = 0x00FFFFFFu;
-        const uint32_t total = n0 * n1;
+        const uint32_t total = n0 * n1;                            // <= 2^14: the float quotient is exact
+        const float inv1 = 1.0f / (float)n1;
         for (uint32_t t = lane; t < total && !stop; t += 32) {
-          const uint32_t t0 = t / n1;
+          const uint32_t t0 = (uint32_t)(((float)t + 0.5f) * inv1);
           const uint32_t e0 = entries[t0], e1 = entries[128u + t - t0 * n1];
           if (((e0 ^ e1) & shared1) != 0u) continue;
           const uint32_t p = ((e0 | e1) & kLp) | (e0 & e1 & ~kLp);
