@@ -84,13 +84,13 @@ struct Found {
 struct LdcaRead {
   const uint32_t* bits;
   const uint4* stamps;
-  ActiveIds ids;
+  uint32_t cur4, k4;
 };
 
 template <bool kSliding>
 __device__ __forceinline__ uint32_t ldc_word(const LdcaRead& a, uint64_t w) {
   if (!kSliding) return a.bits[w];
-  return a.bits[w] | active32(a.stamps[2 * w], a.stamps[2 * w + 1], a.ids);
+  return a.bits[w] | active32(a.stamps[2 * w], a.stamps[2 * w + 1], a.cur4, a.k4);
 }
 
 // word index of the first word of host ip's LDC line in LDCA row i
@@ -237,7 +237,10 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
          uint32_t k_slices, uint32_t z_theta, Found f) {
   constexpr bool kStaged = kForm != Form::kDirect;
   extern __shared__ __align__(16) uint32_t s_dyn[];
-  if (kSliding) ldca.ids = active_ids((uint32_t)(*clock % 255u) + 1u, k_slices);   // the router's current window
+  if (kSliding) {                                   // the window of the router's current slice
+    ldca.cur4 = ((uint32_t)(*clock % 255u) + 1u) * 0x01010101u;
+    ldca.k4 = k_slices * 0x01010101u;
+  }
   __shared__ uint32_t s_queue_n[kDetectWarps], s_next;
   __shared__ uint64_t s_pending[kDetectWarps][kPending];
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
@@ -691,7 +694,7 @@ cudaError_t detect_launch(const DevParams& d, const uint8_t* seav, const LdcaRea
 cudaError_t launch_detect(const DevParams& d, const uint8_t* seav, const uint32_t* ldca,
                           uint32_t z_theta, uint64_t* keys, uint32_t cap, uint64_t max_join,
                           DetectStatus* status, cudaStream_t s) {
-  return detect_launch<false>(d, seav, LdcaRead{ldca, nullptr, {}}, nullptr, 0u, z_theta, keys, cap, max_join,
+  return detect_launch<false>(d, seav, LdcaRead{ldca, nullptr, 0u, 0u}, nullptr, 0u, z_theta, keys, cap, max_join,
                               status, s);
 }
 
@@ -699,7 +702,7 @@ cudaError_t launch_detect_sliding(const DevParams& d, const uint8_t* seav, const
                                   const uint8_t* st_ldca, const uint64_t* clock, uint32_t k, uint32_t z_theta,
                                   uint64_t* keys, uint32_t cap, uint64_t max_join, DetectStatus* status,
                                   cudaStream_t s) {
-  const LdcaRead a{ldca, reinterpret_cast<const uint4*>(st_ldca), {}};
+  const LdcaRead a{ldca, reinterpret_cast<const uint4*>(st_ldca), 0u, 0u};
   return detect_launch<true>(d, seav, a, clock, k, z_theta, keys, cap, max_join, status, s);
 }
 

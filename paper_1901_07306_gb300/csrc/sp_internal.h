@@ -157,47 +157,28 @@ struct FoldSrcs {
 cudaError_t launch_fold_multi(const DevParams& d, const FoldSrcs& src, uint32_t* ldca, int grid, cudaStream_t st,
                               const uint32_t* fresh);
 // Sliding window stamps (Sec. 5.2): one byte per bit holding the id of the
-// last slice that set it, id(t) = t mod 255 + 1 (0 = never set).  The ids of
-// the window's k slices (k <= 128) that end at cur are, in bytes mod 256, the k
-// values from lo = cur - k + 1 on, or, where the window reaches back past id 1,
-// the k + 1 values from lo = 256 - (k - cur) to cur, among them 0, which is no
-// id.  So a stamp s is active iff s != 0 and (s - lo mod 256 < k or s == cur);
-// four stamps at a time, in plain word arithmetic (the byte-wise SIMD
-// intrinsics, which this GPU emulates, took about twice the instructions: the
-// window pass over profile D's SEAV 24 us, this way WINFIG).
-struct ActiveIds {
-  uint32_t sub7, not_lo7, k4, cur4;       // lo without its top bits, the inverse of its top bits, k, cur
-};
-__device__ __forceinline__ ActiveIds active_ids(uint32_t cur, uint32_t k) {
-  const uint32_t lo4 = (cur >= k ? cur - k + 1u : 256u - (k - cur)) * 0x01010101u;
-  return ActiveIds{lo4 & 0x7F7F7F7Fu, ~lo4 & 0x80808080u, k * 0x01010101u, cur * 0x01010101u};
+// last slice that set it, id(t) = t mod 255 + 1 (0 = never set).  Byte j of
+// active_mask4 is 0xFF iff byte j of s is an active stamp: non-zero, of age
+// (cur - stamp) mod 255 below k (byte-wise SIMD: d = cur - s mod 256, and
+// age = d - 1 where cur < s, the mod-255 wrap).  cur4 and k4 hold cur and k
+// in every byte (k <= 128).
+__device__ __forceinline__ uint32_t active_mask4(uint32_t s, uint32_t cur4, uint32_t k4) {
+  const uint32_t d = __vsub4(cur4, s);
+  const uint32_t age = __vadd4(d, __vcmpltu4(cur4, s));       // + 0xFF = - 1 where cur < s
+  return __vcmpltu4(age, k4) & ~__vcmpeq4(s, 0u);
 }
 
-// Bit 7 of byte j is set iff byte j of s is an active stamp; all other bits are 0.
-__device__ __forceinline__ uint32_t active_high4(uint32_t s, const ActiveIds& a) {
-  constexpr uint32_t kHigh = 0x80808080u, kLow = 0x7F7F7F7Fu;
-  const uint32_t d = ((s | kHigh) - a.sub7) ^ ((s ^ a.not_lo7) & kHigh);   // s - lo, byte by byte
-  const uint32_t ge = (d | kHigh) - a.k4;                                  // bit 7: the low bits of d >= k
-  const uint32_t x = s ^ a.cur4;
-  const uint32_t other = ((x & kLow) + kLow) | x;                          // bit 7: s != cur
-  const uint32_t set = ((s & kLow) + kLow) | s;                            // bit 7: s != 0
-  return (~(ge | d) | ~other) & set & kHigh;
+// The same test as 4 bits (bit j for byte j): the four partial products of
+// the multiply land on distinct bits 21..24, so nothing carries.
+__device__ __forceinline__ uint32_t active4(uint32_t s, uint32_t cur4, uint32_t k4) {
+  return (((active_mask4(s, cur4, k4) & 0x01010101u) * 0x00204081u) >> 21) & 0xFu;
 }
 
-// Byte j is 0xFF iff byte j of s is an active stamp.
-__device__ __forceinline__ uint32_t active_mask4(uint32_t s, const ActiveIds& a) {
-  return (active_high4(s, a) >> 7) * 0xFFu;
-}
-
-// The 32 active bits of one sketch word from its 32 stamps (two uint4).  The
-// product moves the four bits of a group to the top, where nothing carries into
-// them, and the funnel shift takes them over.
-__device__ __forceinline__ uint32_t active32(const uint4& a, const uint4& b, const ActiveIds& ids) {
-  const uint32_t v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-  uint32_t out = 0;
-#pragma unroll
-  for (int q = 7; q >= 0; --q) out = __funnelshift_l(active_high4(v[q], ids) * 0x00204081u, out, 4);
-  return out;
+// The 32 active bits of one sketch word from its 32 stamps (two uint4).
+__device__ __forceinline__ uint32_t active32(const uint4& a, const uint4& b, uint32_t cur4, uint32_t k4) {
+  return active4(a.x, cur4, k4) | active4(a.y, cur4, k4) << 4 | active4(a.z, cur4, k4) << 8 |
+         active4(a.w, cur4, k4) << 12 | active4(b.x, cur4, k4) << 16 | active4(b.y, cur4, k4) << 20 |
+         active4(b.z, cur4, k4) << 24 | active4(b.w, cur4, k4) << 28;
 }
 
 // sliding window (sp_slide.cu); a sketch region is nw 32-bit words, word i

@@ -55,12 +55,13 @@ __global__ void __launch_bounds__(kThreads)
 k_clean(uint4* __restrict__ st, uint64_t units16, const uint64_t* __restrict__ clock, uint32_t k) {
   const uint64_t t = *clock, M = 255u - k, seg = t % M;
   const uint64_t lo16 = units16 * seg / M, hi16 = units16 * (seg + 1) / M;
-  const ActiveIds ids = active_ids((uint32_t)(t % 255u) + 1u, k);
+  const uint32_t cur = (uint32_t)(t % 255u) + 1u;
+  const uint32_t cur4 = cur * 0x01010101u, k4 = k * 0x01010101u;
   for (uint64_t i = lo16 + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < hi16;
        i += (uint64_t)gridDim.x * blockDim.x) {
     const uint4 v = st[i];
-    const uint4 o = make_uint4(v.x & active_mask4(v.x, ids), v.y & active_mask4(v.y, ids),
-                               v.z & active_mask4(v.z, ids), v.w & active_mask4(v.w, ids));
+    const uint4 o = make_uint4(v.x & active_mask4(v.x, cur4, k4), v.y & active_mask4(v.y, cur4, k4),
+                               v.z & active_mask4(v.z, cur4, k4), v.w & active_mask4(v.w, cur4, k4));
     if (o.x != v.x || o.y != v.y || o.z != v.z || o.w != v.w) st[i] = o;
   }
 }
@@ -125,8 +126,7 @@ k_commit_window(uint32_t* __restrict__ seav, uint4* __restrict__ st_seav, uint64
                 uint32_t* __restrict__ ldca, uint4* __restrict__ st_ldca, uint64_t ldca_words,
                 uint32_t* __restrict__ wseav, uint32_t* __restrict__ wldca, const uint64_t* __restrict__ clock,
                 uint32_t k) {
-  const uint32_t id4 = slice_id(clock) * 0x01010101u;
-  const ActiveIds ids = active_ids(slice_id(clock), k);
+  const uint32_t id4 = slice_id(clock) * 0x01010101u, k4 = k * 0x01010101u;   // k <= 128 < 256
   const uint64_t n = seav_words + ldca_words;
   for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x) {
     const bool in_seav = j < seav_words;
@@ -144,7 +144,10 @@ k_commit_window(uint32_t* __restrict__ seav, uint4* __restrict__ st_seav, uint64
       stamp_word(bits, v, id4);
       store8(st, i, v);
     }
-    w[i] = active32(make_uint4(v[0], v[1], v[2], v[3]), make_uint4(v[4], v[5], v[6], v[7]), ids);
+    uint32_t out = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) out |= active4(v[q], id4, k4) << (4 * q);
+    w[i] = out;
   }
 }
 
