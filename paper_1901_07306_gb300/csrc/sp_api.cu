@@ -530,7 +530,7 @@ static void set_binned_shape(sp_ctx* ctx, int index) {
   ctx->bs.shape = sp::binned_shape(index);
   ctx->bs_shape_index = (uint32_t)index;
   ctx->bs.ctas = (uint32_t)sp::binned_ctas(ctx->bs.shape);
-  const uint64_t per_list = ctx->bs.list_words / ((uint64_t)(1u << ctx->p.k_log2) * ctx->bs.ctas);
+  const uint64_t per_list = ctx->bs.list_words / ((uint64_t)sp::kBinRows * ctx->bs.ctas);
   ctx->bs.cap_alloc = (uint32_t)((per_list > 0xFFFFFFF8ull ? 0xFFFFFFF8ull : per_list) & ~7ull);
 }
 
@@ -538,21 +538,21 @@ static int ensure_binned(sp_ctx* ctx, uint32_t router) {
   if (!ctx->bs.lists) {
     ctx->bs.max_pairs = kBinnedRoundPairs;
     ctx->bs.fold_grid = sp::binned_fold_grid();
-    const uint32_t bins = 1u << ctx->p.k_log2;
+    constexpr uint64_t rows = sp::kBinRows;
     // room for the largest round of every shape: max_pairs split into host staging chunks
     const uint32_t chunks = (uint32_t)((ctx->bs.max_pairs + kStagingPairs - 1) / kStagingPairs);
     uint64_t words = 0, max_ctas = 0;
     for (int i = 0; i < sp::binned_shape_count(); ++i) {
       const sp::BinShape h = sp::binned_shape(i);
       const uint64_t ctas = (uint64_t)sp::binned_ctas(h);
-      const uint64_t w = (uint64_t)bins * ctas * sp::binned_list_cap(ctx->bs.max_pairs, bins, h, (uint32_t)ctas, chunks);
+      const uint64_t w = rows * ctas * sp::binned_list_cap(ctx->bs.max_pairs, h, (uint32_t)ctas, chunks);
       if (w > words) words = w;
       if (ctas > max_ctas) max_ctas = ctas;
     }
     if (words >= (1ull << 32)) return SP_ERR_PARAM;   // 32-bit list slots
     ctx->bs.list_words = words;
     if (cudaMalloc(&ctx->bs.lists, words * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMalloc(&ctx->bs.counts, (uint64_t)bins * max_ctas * sizeof(uint32_t)) != cudaSuccess) {
+        cudaMalloc(&ctx->bs.counts, rows * max_ctas * sizeof(uint32_t)) != cudaSuccess) {
       cudaGetLastError();
       cudaFree(ctx->bs.lists);
       ctx->bs.lists = nullptr;
@@ -733,7 +733,6 @@ int sp_update_host(sp_ctx* ctx, uint32_t router, const uint32_t* host_pairs, uin
   const bool binned = use_binned(ctx, n_pairs);
   if (binned && (rc = ensure_binned(ctx, router)) != SP_OK) return rc;
   ctx->slice_dirty[router] = true;
-  const uint32_t bins = 1u << ctx->p.k_log2;
   // Chunks of the host stream go through two device staging buffers: the copy
   // of chunk j + 1 (copy stream) overlaps the scan of chunk j (main stream);
   // ev_free[b] marks the last scan that reads buffer b.  A binned update bins
@@ -745,7 +744,7 @@ int sp_update_host(sp_ctx* ctx, uint32_t router, const uint32_t* host_pairs, uin
     const uint64_t round_n = binned ? ((n_pairs - done) < round_cap ? (n_pairs - done) : round_cap)
                                     : (n_pairs - done);
     const uint32_t chunks = (uint32_t)((round_n + kStagingPairs - 1) / kStagingPairs);
-    const uint32_t cap = binned ? sp::binned_list_cap(round_n, bins, ctx->bs.shape, ctx->bs.ctas, chunks) : 0u;
+    const uint32_t cap = binned ? sp::binned_list_cap(round_n, ctx->bs.shape, ctx->bs.ctas, chunks) : 0u;
     const sp::BinnedScratch s = binned ? binned_scratch(ctx, router) : sp::BinnedScratch();
     uint64_t rdone = 0, rot = 0;
     for (uint32_t c = 0; rdone < round_n; ++c, ++j) {
@@ -872,7 +871,6 @@ int sp_update_batched(sp_ctx* ctx, uint32_t n_batches, const uint32_t* routers,
   }
   for (uint32_t r = 0; r < R; ++r)
     if (total[r]) ctx->slice_dirty[r] = true;
-  const uint32_t bins = 1u << ctx->p.k_log2;
   std::vector<sp_batch> rest;
   rest.reserve(n_batches);
   for (uint32_t r = 0; r < R; ++r) {
@@ -900,13 +898,13 @@ int sp_update_batched(sp_ctx* ctx, uint32_t n_batches, const uint32_t* routers,
       uint64_t sum = 0;
       while (j < mine.size() && sum + n_pairs[mine[j]] <= ctx->bs.max_pairs) {
         const uint32_t l = (uint32_t)((j + 1 - i + sp::kBinMaxSrc - 1) / sp::kBinMaxSrc) + 1;   // + 1: ragged tiles
-        if (j > i && sp::binned_list_cap(sum + n_pairs[mine[j]], bins, ctx->bs.shape, ctx->bs.ctas, l) >
+        if (j > i && sp::binned_list_cap(sum + n_pairs[mine[j]], ctx->bs.shape, ctx->bs.ctas, l) >
                          ctx->bs.cap_alloc) break;
         sum += n_pairs[mine[j++]];
       }
       // the round's batches, up to kBinMaxSrc streams per binning launch
       const uint32_t launches = (uint32_t)((j - i + sp::kBinMaxSrc - 1) / sp::kBinMaxSrc) + 1;
-      const uint32_t cap = sp::binned_list_cap(sum, bins, ctx->bs.shape, ctx->bs.ctas, launches);
+      const uint32_t cap = sp::binned_list_cap(sum, ctx->bs.shape, ctx->bs.ctas, launches);
       const sp::BinnedScratch s = binned_scratch(ctx, r);
       uint64_t rot = 0;
       for (size_t q0 = i; q0 < j; q0 += sp::kBinMaxSrc) {

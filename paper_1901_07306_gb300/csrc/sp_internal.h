@@ -57,6 +57,9 @@ __host__ __device__ __forceinline__ uint32_t gather_idx(uint32_t lp, uint32_t is
   return (uint32_t)(twice >> isb) & ((1u << ibn) - 1u);
 }
 
+// Staging rows of k_bin, whatever k: H3's hash selects one by its top bits.
+constexpr uint32_t kBinRowsLog2 = 10, kBinRows = 1u << kBinRowsLog2;
+
 // Up to kBinMaxSrc streams of one router, binned by one k_bin launch.
 constexpr int kBinMaxSrc = 128;       // a multiple of 32
 struct BinSrc {
@@ -80,8 +83,8 @@ BinShape binned_shape(int i);   // i in [0, binned_shape_count()); 0 is the defa
 
 // Scratch of the binned scan (sp_scan_binned.cu), shared by a context's routers.
 struct BinnedScratch {
-  uint32_t* lists = nullptr;    // [bins][ctas][cap] hips
-  uint32_t* counts = nullptr;   // [bins][ctas]
+  uint32_t* lists = nullptr;    // [kBinRows][ctas][cap] hips; a plane's lists are consecutive
+  uint32_t* counts = nullptr;   // [kBinRows][ctas]
   uint32_t* planes = nullptr;   // plane accumulator of one router, [ceil(W / 8)][k][8] words, W = LR * LC / 32
   bool accumulate = false;      // planes hold earlier bits (load instead of zero)
   BinShape shape{};             // staging shape of the launches
@@ -115,7 +118,7 @@ cudaError_t launch_scan_multi(const DevParams& d, uint8_t* sketches, uint64_t st
 int multi_max_grid(int threads);
 bool binned_applicable(const DevParams& d);
 // list capacity for a round of n_pairs binned by `chunks` launches of a shape
-uint32_t binned_list_cap(uint64_t n_pairs, uint32_t bins, const BinShape& shape, uint32_t ctas, uint32_t chunks);
+uint32_t binned_list_cap(uint64_t n_pairs, const BinShape& shape, uint32_t ctas, uint32_t chunks);
 uint32_t binned_tile_pairs(const BinShape& shape);
 // bytes of one router's plane accumulator ([ceil(W / 8)][k][8] words)
 uint64_t binned_planes_bytes(const DevParams& d);

@@ -88,7 +88,11 @@ __device__ __forceinline__ void st_chunk(uint32_t* dst, uint4 a, uint4 b) {
 // thread holds kVec 16-byte loads (2 pairs each) of a tile in registers and
 // issues the loads of tile i + 1 before it works on tile i, so the copy from
 // HBM overlaps the work.  What is left after whole rounds over the blocks is
-// cut into one small tile for each block.  Every bin owns a staging
+// cut into one small tile for each block.  H3's hash selects one of 1,024
+// rows by its top 10 bits, so that rows fill alike for every k: with k < 1024 a
+// bin (the hash's top log2 k bits) has several rows and lists, consecutive ones
+// (k = 256 with a row per bin: 64 arrivals per 44-hip row and round, and 2^23
+// pairs took 136 us, so 61).  Every row is a staging
 // row of STAGE hips in shared memory that persists across tiles (a
 // write-combining buffer for the bin's list).  Per tile:
 //   1. every thread hashes its pairs, queues the sampled pairs (Sec. 3.1) for
@@ -113,7 +117,7 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
   constexpr int TILE = QUADS * 2;
   constexpr int QUEUE = TPR * TILE / 32;              // sampled pairs per round: 4x the expected 2^-7
   extern __shared__ __align__(128) uint8_t smem_raw[];
-  const uint32_t bins = 1u << d.k_log2;                                // <= 1024
+  constexpr uint32_t bins = kBinRows;                                  // rows; bin b has kBinRows / k of them
   uint32_t* stage = reinterpret_cast<uint32_t*>(smem_raw);             // [bins][STAGE], then a 32-word sink
   uint32_t* sink = stage + bins * STAGE;                                // stores of pairs a full row refused
   uint2* s_queue = reinterpret_cast<uint2*>(sink + 32);               // [QUEUE] sampled (hip, h1)
@@ -126,14 +130,15 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
   const uint32_t G = gridDim.x, cta = blockIdx.x;
   const uint32_t slot = (cta + rot) % G;          // which tiles this block takes
   const uint32_t tau_mask = (1u << d.tau) - 1u;
-  const uint32_t h3_shift = 32u - d.k_log2;
+  constexpr uint32_t h3_shift = 32u - kBinRowsLog2;
+  const uint32_t row_shift = kBinRowsLog2 - d.k_log2;                   // bin of a row
   const uint32_t lane = tid & 31u;
   uint32_t lt_mask;                                // lanes below this one
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt_mask));
   // a hip whose row or list was full: its LDCA bits go straight to L2, and
   // the router's flag tells the fold that the LDCA is no longer all zero
-  auto spill = [&](uint32_t hip, uint32_t b) {
-    ldca_red(d, ldca, hip, b);
+  auto spill = [&](uint32_t hip, uint32_t b) {     // b: the row
+    ldca_red(d, ldca, hip, b >> row_shift);
     if (ovf) *ovf = 1u;
   };
   // A stream is a body of 16-byte quads (two pairs) and up to two single
@@ -749,8 +754,8 @@ k_fold8(FoldSrcs src, uint32_t* ldca, uint32_t W, uint32_t k_log2, const uint32_
 template <int THREADS, int STAGE, int TPR, int PER_SM>
 cudaError_t bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, const BinSrc& src,
                       const BinnedScratch& s, uint32_t cap, bool append, uint32_t rot, cudaStream_t st) {
-  const uint32_t bins = 1u << d.k_log2;
-  // the bins' staging rows, the sampled-pair queue, the full rows' pairs, 2 counters per bin
+  constexpr uint32_t bins = kBinRows;
+  // the staging rows, the sampled-pair queue, the full rows' pairs, 2 counters per row
   const size_t bin_smem = (size_t)bins * STAGE * 4 + 32 * 4 + (size_t)(TPR * THREADS * kVec * 2 / 32 + 2 * kOver) * 8 +
                           (size_t)bins * 8;
   auto kern = k_bin<THREADS, STAGE, TPR, PER_SM>;
@@ -788,7 +793,8 @@ template <int LR, int THREADS, int LCL, int SPLIT = 1>
 cudaError_t apply_round_t(const DevParams& d, const BinnedScratch& s, uint32_t cap, bool accumulate, cudaStream_t st) {
   const uint32_t bins = 1u << d.k_log2;
   const uint32_t chunks = ((((uint32_t)(LR / SPLIT) << d.lc_log2) >> 5) + 7u) / 8u;
-  const size_t apply_smem = ((size_t)chunks * 8u + s.ctas) * sizeof(uint32_t);   // the rows, the lists' counts
+  const uint32_t n_lists = s.ctas << (kBinRowsLog2 - d.k_log2);                    // of a plane
+  const size_t apply_smem = ((size_t)chunks * 8u + n_lists) * sizeof(uint32_t);    // the rows, the lists' counts
   auto kern = k_apply<LR, THREADS, LCL, SPLIT>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem);
   if (e != cudaSuccess) return e;
@@ -797,7 +803,7 @@ cudaError_t apply_round_t(const DevParams& d, const BinnedScratch& s, uint32_t c
   while (chunks % box != 0u) --box;
   CUtensorMap map;
   if ((e = plane_map(s.planes, bins, chunks * (uint32_t)SPLIT, box, &map)) != cudaSuccess) return e;
-  kern<<<bins * SPLIT, THREADS, apply_smem, st>>>(d, s.lists, s.counts, s.ctas, cap, s.planes, map, box, accumulate);
+  kern<<<bins * SPLIT, THREADS, apply_smem, st>>>(d, s.lists, s.counts, n_lists, cap, s.planes, map, box, accumulate);
   return cudaGetLastError();
 }
 
@@ -841,13 +847,13 @@ BinShape binned_shape(int i) { return kShapes[(i >= 0 && i < binned_shape_count(
 
 // List capacity for a round of n_pairs split into `chunks` binning launches:
 // a block takes at most ceil(tiles / ctas) + 1 tiles per launch (the tile to
-// block mapping rotates between launches), spread over the bins; 8 standard
+// block mapping rotates between launches), spread over the rows; 8 standard
 // deviations plus 32 of headroom, so that only skewed inputs overflow.
-uint32_t binned_list_cap(uint64_t n_pairs, uint32_t bins, const BinShape& shape, uint32_t ctas, uint32_t chunks) {
+uint32_t binned_list_cap(uint64_t n_pairs, const BinShape& shape, uint32_t ctas, uint32_t chunks) {
   const uint64_t tile = binned_tile_pairs(shape);
   const uint64_t tiles = (n_pairs + tile - 1) / tile;
   const uint64_t per_cta = (tiles + ctas - 1) / ctas + (chunks > 1 ? chunks : 1);
-  const double m = (double)(per_cta * tile < n_pairs ? per_cta * tile : n_pairs) / bins;
+  const double m = (double)(per_cta * tile < n_pairs ? per_cta * tile : n_pairs) / kBinRows;
   uint64_t cap = (uint64_t)(m + 8.0 * sqrt(m + 1.0) + 32.0);
   cap = (cap + 7) & ~7ull;                                   // 32-byte list starts
   return (uint32_t)cap;
@@ -945,7 +951,7 @@ cudaError_t launch_scan_binned(const DevParams& d, uint8_t* seav, uint32_t* ldca
   bool accumulate = s.accumulate;
   while (done < n_pairs) {
     const uint64_t n = (n_pairs - done) < s.max_pairs ? (n_pairs - done) : s.max_pairs;
-    const uint32_t cap = binned_list_cap(n, 1u << d.k_log2, s.shape, s.ctas, 1);
+    const uint32_t cap = binned_list_cap(n, s.shape, s.ctas, 1);
     BinSrc src = bin_src_one(pairs + 2 * done, n);
     uint64_t rot = 0;
     cudaError_t e = binned_bin_chunk(d, seav, ldca, src, s, cap, false, &rot, st);
