@@ -29,7 +29,7 @@ constexpr uint64_t kBinnedRoundPairs = 1ull << 26;  // pairs per binning round
 // copies, so after the last copy only one round of 2^24 pairs is left to apply.
 constexpr uint64_t kHostRoundPairs = 1ull << 24;
 constexpr uint32_t kResultPrefix = 2048;            // records fetched with the status (48 KiB)
-constexpr size_t kKerrAt = 64, kRecordsAt = 128;    // result block: status, error word, records
+constexpr size_t kKerrAt = 64, kTicketAt = 96, kRecordsAt = 128;    // result block: status, error word, batch ticket, records
 constexpr uint32_t kDefaultTimeoutMs = 60000;       // bound of every wait on the stream
 constexpr uint64_t kAlign = 256;
 
@@ -97,6 +97,7 @@ struct sp_ctx {
   uint8_t* results = nullptr;
   DetectStatus* published() const { return reinterpret_cast<DetectStatus*>(results); }
   uint32_t* kerr() const { return reinterpret_cast<uint32_t*>(results + kKerrAt); }
+  uint32_t* ticket() const { return reinterpret_cast<uint32_t*>(results + kTicketAt); }   // of k_scan_multi
   sp_candidate* records() const { return reinterpret_cast<sp_candidate*>(results + kRecordsAt); }
   DetectStatus* status = nullptr;           // the running detect's; zero between detects
   bool status_clean = true;                 // false: a detect's second launch failed
@@ -828,7 +829,7 @@ static int launch_table(sp_ctx* ctx, const sp_batch* dev_tab, uint32_t n) {
   for (uint32_t i = 0; i < n; i += kMaxTable) {
     const uint32_t m = (n - i) < kMaxTable ? (n - i) : kMaxTable;
     if (sp::launch_scan_multi(ctx->d, ctx->sketches, ctx->stride, ctx->seav_pad, ctx->p.n_routers, dev_tab + i, m,
-                              ctx->kerr(), ctx->multi_threads, ctx->multi_grid, ctx->stream) != cudaSuccess)
+                              ctx->kerr(), ctx->ticket(), ctx->multi_threads, ctx->multi_grid, ctx->stream) != cudaSuccess)
       return SP_ERR_CUDA;
   }
   return SP_OK;

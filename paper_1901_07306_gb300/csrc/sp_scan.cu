@@ -192,15 +192,21 @@ int grid_for() {
 // The work unit is a chunk of kChunk pairs of one batch.  Every block scans
 // the batch table once into a shared prefix of chunk counts (a batch with a
 // router out of range or a misaligned stream counts 0 chunks and raises bit 1
-// of *err), then takes chunks g = block, block + grid, ... and finds each
-// chunk's batch by binary search.  Routers index the context's sketches.
+// of *err), then takes the next chunk of the table by a ticket, fetched while
+// the chunk before is scanned, and finds the chunk's batch by binary search.
+// Routers index the context's sketches.  Tickets keep the chunks in flight next
+// to each other in the table, whose batches the host groups by router: with
+// chunks block, block + grid, ... the blocks drifted apart until the REDs went to
+// more sketches than L2 holds and nearly each one missed (15 routers of profile
+// D x 2.7 M uniform pairs: 4,226 us, 1,662 with tickets).  A chunk draws one
+// ticket, so the drawer of the last one zeroes the counter for the next launch.
 constexpr uint32_t kChunk = 2048;
 
 template <int LR, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 k_scan_multi(DevParams d, uint8_t* __restrict__ sketches, uint64_t stride, uint64_t seav_pad,
              uint32_t n_routers, const sp_batch* __restrict__ desc, uint32_t n_batches,
-             uint32_t* __restrict__ err) {
+             uint32_t* __restrict__ err, uint32_t* __restrict__ ticket) {
   extern __shared__ uint64_t s_pref[];                     // [n_batches + 1]
   __shared__ uint64_t s_carry;
   const uint32_t tid = threadIdx.x;
@@ -231,8 +237,15 @@ k_scan_multi(DevParams d, uint8_t* __restrict__ sketches, uint64_t stride, uint6
     if (tid == THREADS - 1) s_carry += s_tmp[tid];
     __syncthreads();
   }
-  const uint64_t total = s_pref[n_batches];
-  for (uint64_t g = blockIdx.x; g < total; g += gridDim.x) {
+  const uint64_t total = s_pref[n_batches];               // < 2^32 chunks
+  __shared__ uint32_t s_next[2];
+  uint32_t g = blockIdx.x;                                 // the first chunk; then gridDim.x + ticket
+  for (uint32_t turn = 0; g < total; turn ^= 1u) {
+    if (tid == 0) {
+      const uint32_t t = atomicAdd(ticket, 1u);            // one per chunk
+      if (t == (uint32_t)total - 1u) *ticket = 0u;
+      s_next[turn] = gridDim.x + t;
+    }
     uint32_t lo = 0, hi = n_batches;                       // last b with s_pref[b] <= g
     while (hi - lo > 1) {
       const uint32_t mid = (lo + hi) >> 1;
@@ -248,25 +261,28 @@ k_scan_multi(DevParams d, uint8_t* __restrict__ sketches, uint64_t stride, uint6
       const uint2 v = __ldcs(p2 + i);
       scan_pair<LR>(d, seav, ldca, v.x, v.y, tau_mask);
     }
+    __syncthreads();
+    g = s_next[turn];
   }
 }
 
 template <int LR>
 cudaError_t multi_lr(const DevParams& d, uint8_t* sketches, uint64_t stride, uint64_t seav_pad, uint32_t n_routers,
-                     const sp_batch* desc, uint32_t n_batches, uint32_t* err, int threads, int grid, cudaStream_t s) {
+                     const sp_batch* desc, uint32_t n_batches, uint32_t* err, uint32_t* ticket, int threads, int grid,
+                     cudaStream_t s) {
   const size_t smem = ((size_t)n_batches + 1) * sizeof(uint64_t);
   switch (threads) {
     case 128:
       cudaFuncSetAttribute(k_scan_multi<LR, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_scan_multi<LR, 128><<<grid, 128, smem, s>>>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err);
+      k_scan_multi<LR, 128><<<grid, 128, smem, s>>>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket);
       break;
     case 512:
       cudaFuncSetAttribute(k_scan_multi<LR, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_scan_multi<LR, 512><<<grid, 512, smem, s>>>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err);
+      k_scan_multi<LR, 512><<<grid, 512, smem, s>>>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket);
       break;
     default:
       cudaFuncSetAttribute(k_scan_multi<LR, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      k_scan_multi<LR, 256><<<grid, 256, smem, s>>>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err);
+      k_scan_multi<LR, 256><<<grid, 256, smem, s>>>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket);
       break;
   }
   return cudaGetLastError();
@@ -276,17 +292,17 @@ cudaError_t multi_lr(const DevParams& d, uint8_t* sketches, uint64_t stride, uin
 
 cudaError_t launch_scan_multi(const DevParams& d, uint8_t* sketches, uint64_t stride, uint64_t seav_pad,
                               uint32_t n_routers, const sp_batch* desc, uint32_t n_batches, uint32_t* err,
-                              int threads, int grid, cudaStream_t s) {
+                              uint32_t* ticket, int threads, int grid, cudaStream_t s) {
   if (n_batches == 0) return cudaSuccess;
   switch (d.lr) {
-    case 1: return multi_lr<1>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, threads, grid, s);
-    case 2: return multi_lr<2>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, threads, grid, s);
-    case 3: return multi_lr<3>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, threads, grid, s);
-    case 4: return multi_lr<4>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, threads, grid, s);
-    case 5: return multi_lr<5>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, threads, grid, s);
-    case 6: return multi_lr<6>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, threads, grid, s);
-    case 7: return multi_lr<7>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, threads, grid, s);
-    default: return multi_lr<8>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, threads, grid, s);
+    case 1: return multi_lr<1>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket, threads, grid, s);
+    case 2: return multi_lr<2>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket, threads, grid, s);
+    case 3: return multi_lr<3>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket, threads, grid, s);
+    case 4: return multi_lr<4>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket, threads, grid, s);
+    case 5: return multi_lr<5>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket, threads, grid, s);
+    case 6: return multi_lr<6>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket, threads, grid, s);
+    case 7: return multi_lr<7>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket, threads, grid, s);
+    default: return multi_lr<8>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket, threads, grid, s);
   }
 }
 
