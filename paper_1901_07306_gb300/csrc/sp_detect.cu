@@ -10,8 +10,8 @@
 //      its SEs falls below weight 3 -- AND only clears bits, so the pruning
 //      loses nothing against testing complete tuples (Sec. 3.2, SEU test).
 //   3. A complete tuple fixes every LP bit (Eq. 3, coverage constraint);
-//      ip = LP << r | RP goes to a per-warp queue.  When the SEA is done the
-//      warp tests the queued hosts together: the LDC union (AND over the LR
+//      ip = LP << r | RP goes to a per-warp queue.  Once enough are queued, or
+//      the warp has no SEA left, it tests the queued hosts together: the LDC union (AND over the LR
 //      rows, Sec. 3.3) of one host is read as LR lines of k bits spread over
 //      the lanes (one coalesced load per row and lane), z0 = k - popc by a
 //      warp reduction.  The host survives when z0 <= Z_theta, the integer
@@ -230,7 +230,10 @@ __device__ void test_queue(const DevParams& d, const LdcaRead& ldca, const uint3
 // round trip to the LDC lines per test pass.  The next SEA is copied
 // meanwhile; hosts are tested two a pass once kTestAt are queued or the warp
 // is done, not one or two after every SEA; and the warps of a block take its
-// SEAs from one counter, since SEAs differ.  DETFIG
+// SEAs from one counter, since SEAs differ.  Detect of 16 merged routers (65,536
+// SEAs): 139 us with a test after every SEA and SEAs in a fixed stride, 121 this
+// way, 106 with the four-row form and without spills (five blocks per SM there,
+// 48 registers; six, at 40, gain nothing).
 template <bool kSliding, Form kForm>
 __global__ void __launch_bounds__(kDetectThreads, kForm == Form::kFour ? 5 : 4)
 k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uint64_t* __restrict__ clock,

@@ -10,8 +10,8 @@
 //           issued before the current tile's work), does the SEAV update of
 //           Sec. 3.1-3.2 for sampled pairs (L2 RED, 1 pair in 2^tau), and
 //           stages each hip in a shared-memory row of its bin b; a row's whole
-//           8-hip chunks go to the block's private list for that bin with one
-//           32-byte store each (no global atomics; lists[b][block][0 .. cap)).
+//           8-hip chunks go to the block's private list for that row with one
+//           32-byte store each (no global atomics; lists[row][block][0 .. cap)).
 //           Hips that find their row full wait for the end of the round; only
 //           skewed inputs (a full list, a row that stays full) send hips to L2
 //           REDs instead (any input is correct).
@@ -19,12 +19,13 @@
 //           zero (or from the router's pending plane when earlier updates of
 //           the window have not been folded yet), sets bit (i, LH_i(hip)) for
 //           every listed hip and row i with shared atomic OR, and stores the
-//           plane back (the block owns it).
-//  k_fold   (before the next detect, merge or export of the router) ORs the
-//           plane accumulator into the LDCA's logical layout
-//           [LR][LC][k / 32]: a warp loads word J of 32 consecutive planes and
-//           a 5-stage butterfly of warp shuffles transposes the 32 x 32 bit
-//           block, giving lane t the 32-bit word of LDC 32 J + t.
+//           plane back by TMA (the block owns it).  Bounds: the load-store pipe,
+//           94% busy at 2^26 pairs, by the LR random atomics per hip.
+//  k_fold   (before the next detect, copy or export of the router, or in a
+//           merge, over all sources at once) ORs the plane accumulators into
+//           the LDCA's logical layout [LR][LC][k / 32]: word J of 32 consecutive
+//           planes is a 32 x 32 bit block whose transpose holds the words of LDCs
+//           32 J .. 32 J + 31.
 //
 // Applicable when the bins are the LDC's k bit positions (k <= 1024) and one
 // plane fits in shared memory as whole words (LC >= 32, LR x LC <= 2^20 bits).
