@@ -253,9 +253,9 @@ typedef struct sp_batch {
 /* Batched scan (the WPs of Sec. 4.1 fed together): n_batches
  * (router, pairs, n_pairs) triples of device streams of uneven sizes, given as
  * three host arrays; routers[b] may repeat.  Routers whose batches add up to
- * at least 2^22 pairs take the binned scan (one binning launch per batch, one
- * plane launch per router); all other batches are scanned by ONE persistent
- * launch over a batch table, whose block shape comes from sp_autotune (or a
+ * at least 2^22 pairs take the binned scan (one binning launch per 128
+ * batches, one plane launch per router); all other batches are scanned by ONE
+ * persistent launch over a batch table, whose block shape comes from sp_autotune (or a
  * default).  Same per-batch semantics and errors as sp_update.  A stream may
  * also be page-locked host memory mapped into the device's address space
  * (cudaHostAlloc or cudaHostRegister; under unified addressing the host
