@@ -1123,6 +1123,14 @@ int sp_merge(sp_ctx* ctx, const uint32_t* routers, uint32_t n, uint32_t dst_rout
                                 ldca_known_zero(ctx, r) ? ctx->ovf + r : nullptr});
   }
   if (srcs.empty()) return fold_router(ctx, dst_router);
+  if (ctx->captured && pending) {
+    // a recorded merge leaves every router's bits in its LDCA, where calls
+    // after a replay find them: the host does not see a replay's planes
+    int rc = fold_router(ctx, dst_router);
+    for (uint32_t i = 0; i < n && rc == SP_OK; ++i) rc = fold_router(ctx, routers[i]);
+    if (rc != SP_OK) return rc;
+    pending = false;
+  }
   const uint32_t* fresh = ldca_known_zero(ctx, dst_router) ? ctx->ovf + dst_router : nullptr;
   ctx->ldca_zero[dst_router] = false;
   if (!pending)

@@ -111,3 +111,29 @@ def test_reset_after_graph_replays(sp, torch):  # noqa: F811
             sp.sp_reset(ctx.ctx, 0)
             seav, ldca = ctx.sketch_image(0)
             assert not seav.any() and not ldca.any()
+
+
+def test_recorded_merge_then_calls_on_its_sources(sp, torch):  # noqa: F811
+    """A graph of a binned update and a merge, replayed between resets: the
+    source's bits are found by calls after the replay, not only the merged ones."""
+    kw = dict(BASE, k_log2=8, lr=3, lc_log2=6, n_routers=3, scan_mode=2)
+    op = oracle_params(kw)
+    x, y = _pairs("planes", 4), _pairs("planes", 5)
+    t, u = dev(torch, x), dev(torch, y)
+    with sp.SuperPoint(**kw) as ctx:
+        sp.sp_reserve(ctx.ctx)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            sp.sp_set_stream(ctx.ctx, torch.cuda.current_stream())
+            ctx.update(t, router=0)
+            ctx.merge([0, 2], 1)
+        sp.sp_set_stream(ctx.ctx, torch.cuda.current_stream())
+        for _ in range(2):
+            sp.sp_reset_range(ctx.ctx, 0, 3)
+            ctx.update(u, router=2)                       # pending when the replay merges
+            g.replay()
+            assert_same_sketch(ctx, O.Sketch(op).update(x), 0)
+            assert_same_sketch(ctx, O.Sketch(op).update(y), 2)
+            ctx.merge([0, 2], 1)
+            assert_same_sketch(ctx, O.Sketch(op).update(x).update(y), 1)
