@@ -29,7 +29,8 @@ constexpr uint64_t kBinnedRoundPairs = 1ull << 26;  // pairs per binning round
 // copies, so after the last copy only one round of 2^24 pairs is left to apply.
 constexpr uint64_t kHostRoundPairs = 1ull << 24;
 constexpr uint32_t kResultPrefix = 2048;            // records fetched with the status (48 KiB)
-constexpr size_t kKerrAt = 64, kTicketAt = 96, kRecordsAt = 128;    // result block: status, error word, batch ticket, records
+// result block: status, error word, batch ticket, `pending` before a binned round, records
+constexpr size_t kKerrAt = 64, kTicketAt = 96, kPriorAt = 100, kRecordsAt = 128;
 constexpr uint32_t kDefaultTimeoutMs = 60000;       // bound of every wait on the stream
 constexpr uint64_t kAlign = 256;
 
@@ -98,6 +99,7 @@ struct sp_ctx {
   DetectStatus* published() const { return reinterpret_cast<DetectStatus*>(results); }
   uint32_t* kerr() const { return reinterpret_cast<uint32_t*>(results + kKerrAt); }
   uint32_t* ticket() const { return reinterpret_cast<uint32_t*>(results + kTicketAt); }   // of k_scan_multi
+  uint32_t* prior() const { return reinterpret_cast<uint32_t*>(results + kPriorAt); }     // BinnedScratch::prior
   sp_candidate* records() const { return reinterpret_cast<sp_candidate*>(results + kRecordsAt); }
   DetectStatus* status = nullptr;           // the running detect's; zero between detects
   bool status_clean = true;                 // false: a detect's second launch failed
@@ -120,15 +122,19 @@ struct sp_ctx {
   sp::BinnedScratch bs;
   uint32_t** planes = nullptr;              // [n_routers], lazily allocated
   bool* planes_dirty = nullptr;             // bits not yet folded into the LDCA
+  // a binned update of r was recorded in a stream capture: its replays leave
+  // planes pending that the host knows nothing of, so every later fold is
+  // launched and the device decides (RouterFlags::pending)
+  bool* planes_recorded = nullptr;
   // ldca_zero[r]: since r's last zeroing only binned rounds wrote its LDCA
   // (discrete contexts), so the next fold may write the planes without
   // reading the LDCA -- unless a binning launch spilled a bit past a full
-  // list, which sets the device flag ovf[r] (cleared with the zeroing)
+  // list, which sets flags[r].spilled (cleared with the zeroing)
   bool* ldca_zero = nullptr;
-  uint32_t* ovf = nullptr;
+  sp::RouterFlags* flags = nullptr;         // [n_routers], device
   // set once a call of this context was recorded in a stream capture: a
   // replay writes LDCAs that the host then knows nothing of, so ldca_zero says
-  // nothing any more
+  // nothing any more, and whether planes hold bits is decided on the device
   bool captured = false;
   // sliding window (Sec. 5): one stamp byte per bit, per-router slice clock;
   // the bit sketch of a sliding router holds the current slice's bits until
@@ -350,6 +356,7 @@ void sp_destroy(sp_ctx* ctx) {
     free(ctx->planes);
   }
   free(ctx->planes_dirty);
+  free(ctx->planes_recorded);
   free(ctx->slice);
   cudaFree(ctx->clock);
   free(ctx->slice_dirty);
@@ -363,7 +370,7 @@ void sp_destroy(sp_ctx* ctx) {
   cudaFree(ctx->window);
   cudaFree(ctx->bs.lists);
   cudaFree(ctx->bs.counts);
-  cudaFree(ctx->ovf);
+  cudaFree(ctx->flags);
   free(ctx->ldca_zero);
   cudaFree(ctx->sketches);
   cudaFree(ctx->keys);
@@ -423,7 +430,7 @@ int sp_create(const sp_params* p, void* cuda_stream, sp_ctx** out) {
       cudaMalloc(&c->keys, key_slots * sizeof(uint64_t)) != cudaSuccess ||
       cudaMalloc(&c->results, kRecordsAt + (uint64_t)c->cap * sizeof(sp_candidate)) != cudaSuccess ||
       cudaMalloc(&c->status, sizeof(DetectStatus)) != cudaSuccess ||
-      cudaMalloc(&c->ovf, sizeof(uint32_t) * p->n_routers) != cudaSuccess ||
+      cudaMalloc(&c->flags, sizeof(sp::RouterFlags) * p->n_routers) != cudaSuccess ||
       cudaMalloc(&c->est_table, ((1ull << p->k_log2) + 1) * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     rc = SP_ERR_NOMEM;
@@ -441,7 +448,7 @@ int sp_create(const sp_params* p, void* cuda_stream, sp_ctx** out) {
       free(table);
     }
   }
-  if (rc == SP_OK && sp::launch_zero_flags(c->sketches, c->stride * p->n_routers, c->ovf, p->n_routers, c->stream) !=
+  if (rc == SP_OK && sp::launch_zero_flags(c->sketches, c->stride * p->n_routers, c->flags, p->n_routers, c->stream) !=
                          cudaSuccess)
     rc = SP_ERR_CUDA;
   if (rc == SP_OK && cudaMemsetAsync(c->status, 0, sizeof(DetectStatus), c->stream) != cudaSuccess) rc = SP_ERR_CUDA;
@@ -451,12 +458,13 @@ int sp_create(const sp_params* p, void* cuda_stream, sp_ctx** out) {
     c->multi_grid = sp::multi_max_grid(c->multi_threads);
     c->planes = static_cast<uint32_t**>(calloc(p->n_routers, sizeof(uint32_t*)));
     c->planes_dirty = static_cast<bool*>(calloc(p->n_routers, sizeof(bool)));
+    c->planes_recorded = static_cast<bool*>(calloc(p->n_routers, sizeof(bool)));
     c->ldca_zero = static_cast<bool*>(calloc(p->n_routers, sizeof(bool)));
     if (c->ldca_zero && p->window_slices <= 1)
       for (uint32_t r = 0; r < p->n_routers; ++r) c->ldca_zero[r] = true;
     c->slice = static_cast<uint64_t*>(calloc(p->n_routers, sizeof(uint64_t)));
     c->slice_dirty = static_cast<bool*>(calloc(p->n_routers, sizeof(bool)));
-    if (!c->planes || !c->planes_dirty || !c->slice || !c->slice_dirty || !c->ldca_zero) rc = SP_ERR_NOMEM;
+    if (!c->planes || !c->planes_dirty || !c->planes_recorded || !c->slice || !c->slice_dirty || !c->ldca_zero) rc = SP_ERR_NOMEM;
   }
   if (rc == SP_OK && p->window_slices > 1) {
     c->sliding = true;
@@ -510,16 +518,36 @@ static void note_capture(sp_ctx* ctx) {
 }
 
 // Whether a router's LDCA is known to be all zero but for spilled bits, which
-// its flag ovf[router] announces.
+// its flag `spilled` announces.
 static bool ldca_known_zero(const sp_ctx* ctx, uint32_t router) { return ctx->ldca_zero[router] && !ctx->captured; }
 
-// Folds a router's pending binned-scan planes into its LDCA.
+// Where the device says whether a router's LDCA that is known to be zero
+// holds spilled bits; null when it is not known to be zero.
+static const uint32_t* spilled_if_zero(const sp_ctx* ctx, uint32_t router) {
+  return ldca_known_zero(ctx, router) ? &ctx->flags[router].spilled : nullptr;
+}
+
+// Whether a router's planes may hold bits that its LDCA has not.
+static bool planes_pending(const sp_ctx* ctx, uint32_t router) {
+  return ctx->planes_dirty[router] || ctx->planes_recorded[router];
+}
+
+// A binned round of a router was issued: its planes are pending.
+static void note_planes(sp_ctx* ctx, uint32_t router) {
+  ctx->planes_dirty[router] = true;
+  if (ctx->captured && capturing(ctx->stream)) ctx->planes_recorded[router] = true;
+}
+
+// Folds a router's pending binned-scan planes into its LDCA.  With recorded
+// calls the device decides: a fold that was recorded while planes were pending
+// must not bring back their bits once the window is over.
 static int fold_router(sp_ctx* ctx, uint32_t router) {
-  if (!ctx->planes_dirty[router]) return SP_OK;
-  const uint32_t* fresh = ldca_known_zero(ctx, router) ? ctx->ovf + router : nullptr;
-  if (sp::launch_fold(ctx->d, ctx->planes[router], ctx->ldca(router), ctx->bs.fold_grid, ctx->stream, fresh) !=
-      cudaSuccess)
+  if (!planes_pending(ctx, router)) return SP_OK;
+  uint32_t* pending = ctx->captured ? &ctx->flags[router].pending : nullptr;
+  if (sp::launch_fold(ctx->d, ctx->planes[router], ctx->ldca(router), ctx->bs.fold_grid, ctx->stream,
+                      spilled_if_zero(ctx, router), pending) != cudaSuccess)
     return SP_ERR_CUDA;
+  if (pending && cudaMemsetAsync(pending, 0, sizeof(*pending), ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
   ctx->planes_dirty[router] = false;
   ctx->ldca_zero[router] = false;
   return SP_OK;
@@ -582,7 +610,8 @@ static sp::BinnedScratch binned_scratch(const sp_ctx* ctx, uint32_t router) {
   sp::BinnedScratch s = ctx->bs;
   s.planes = ctx->planes[router];
   s.accumulate = ctx->planes_dirty[router];
-  s.ovf = ctx->ovf + router;
+  s.flags = ctx->flags + router;
+  s.prior = ctx->captured ? ctx->prior() : nullptr;
   return s;
 }
 
@@ -595,7 +624,7 @@ static int do_update(sp_ctx* ctx, uint32_t router, const uint32_t* dev_pairs, ui
     sp::BinnedScratch s = binned_scratch(ctx, router);
     if (sp::launch_scan_binned(ctx->d, ctx->seav(router), ctx->ldca(router), dev_pairs, n_pairs, s,
                                ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
-    ctx->planes_dirty[router] = true;
+    note_planes(ctx, router);
     return SP_OK;
   }
   ctx->ldca_zero[router] = false;
@@ -612,7 +641,7 @@ static int commit(sp_ctx* ctx, uint32_t router) {
   if (rc != SP_OK || !ctx->slice_dirty[router]) return rc;
   if (sp::launch_commit(reinterpret_cast<uint32_t*>(ctx->seav(router)), ctx->st_seav(router), ctx->seav_words(),
                         ctx->ldca(router), ctx->st_ldca(router), ctx->ldca_bytes / 4, ctx->dev_clock(router),
-                        ctx->stream) != cudaSuccess)
+                        &ctx->flags[router].pending, ctx->stream) != cudaSuccess)
     return SP_ERR_CUDA;
   ctx->slice_dirty[router] = false;
   return SP_OK;
@@ -626,7 +655,8 @@ static int commit_window(sp_ctx* ctx, uint32_t router) {
   if (sp::launch_commit_window(reinterpret_cast<uint32_t*>(ctx->seav(router)), ctx->st_seav(router),
                                ctx->seav_words(), ctx->ldca(router), ctx->st_ldca(router), ctx->ldca_bytes / 4,
                                reinterpret_cast<uint32_t*>(ctx->wseav(router)), ctx->wldca(router),
-                               ctx->dev_clock(router), ctx->p.window_slices, ctx->stream) != cudaSuccess)
+                               ctx->dev_clock(router), ctx->p.window_slices, &ctx->flags[router].pending,
+                               ctx->stream) != cudaSuccess)
     return SP_ERR_CUDA;
   ctx->slice_dirty[router] = false;
   return SP_OK;
@@ -643,7 +673,8 @@ static int commit_seav_window(sp_ctx* ctx, uint32_t router) {
   if (sp::launch_commit_window(reinterpret_cast<uint32_t*>(ctx->seav(router)), ctx->st_seav(router),
                                ctx->seav_words(), ctx->ldca(router), ctx->st_ldca(router), 0,
                                reinterpret_cast<uint32_t*>(ctx->wseav(router)), ctx->wldca(router),
-                               ctx->dev_clock(router), ctx->p.window_slices, ctx->stream) != cudaSuccess)
+                               ctx->dev_clock(router), ctx->p.window_slices, &ctx->flags[router].pending,
+                               ctx->stream) != cudaSuccess)
     return SP_ERR_CUDA;
   return SP_OK;
 }
@@ -663,8 +694,8 @@ static int zero_routers(sp_ctx* ctx, uint32_t first, uint32_t count) {
       any = true;
     }
   const cudaError_t e =
-      any ? sp::launch_reset(ctx->sketches, ctx->stride, ctx->seav_pad, first, count, clean, ctx->ovf, ctx->stream)
-          : sp::launch_zero_flags(ctx->seav(first), ctx->stride * count, ctx->ovf + first, count, ctx->stream);
+      any ? sp::launch_reset(ctx->sketches, ctx->stride, ctx->seav_pad, first, count, clean, ctx->flags, ctx->stream)
+          : sp::launch_zero_flags(ctx->seav(first), ctx->stride * count, ctx->flags + first, count, ctx->stream);
   if (e != cudaSuccess) return SP_ERR_CUDA;
   for (uint32_t r = first; r < first + count; ++r) {
     ctx->planes_dirty[r] = false;                // pending planes belong to the old window
@@ -684,7 +715,7 @@ int sp_reset(sp_ctx* ctx, uint32_t router) {
   ctx->slice[router] = 0;
   if (cudaMemsetAsync(ctx->dev_clock(router), 0, sizeof(uint64_t), ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
   if (sp::launch_zero(ctx->st_seav(router), ctx->st_stride, ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
-  if (sp::launch_zero_flags(ctx->seav(router), ctx->stride, ctx->ovf + router, 1, ctx->stream) != cudaSuccess)
+  if (sp::launch_zero_flags(ctx->seav(router), ctx->stride, ctx->flags + router, 1, ctx->stream) != cudaSuccess)
     return SP_ERR_CUDA;
   return SP_OK;
 }
@@ -770,7 +801,7 @@ int sp_update_host(sp_ctx* ctx, uint32_t router, const uint32_t* host_pairs, uin
     if (binned) {
       if (sp::binned_apply_round(ctx->d, s, cap, ctx->planes_dirty[router], ctx->stream) != cudaSuccess)
         return SP_ERR_CUDA;
-      ctx->planes_dirty[router] = true;
+      note_planes(ctx, router);
     }
     done += round_n;
   }
@@ -919,7 +950,7 @@ int sp_update_batched(sp_ctx* ctx, uint32_t n_batches, const uint32_t* routers,
             cudaSuccess) return SP_ERR_CUDA;
       }
       if (sp::binned_apply_round(ctx->d, s, cap, ctx->planes_dirty[r], ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
-      ctx->planes_dirty[r] = true;
+      note_planes(ctx, r);
       i = j;
     }
   }
@@ -1061,7 +1092,7 @@ int sp_autotune_binned(sp_ctx* ctx, const uint32_t* dev_pairs, uint64_t n_pairs,
     const sp::BinnedScratch s = binned_scratch(ctx, 0);
     if (sp::launch_scan_binned(ctx->d, ctx->seav(0), ctx->ldca(0), dev_pairs, n_pairs, s, ctx->stream) != cudaSuccess)
       return SP_ERR_CUDA;
-    ctx->planes_dirty[0] = true;
+    note_planes(ctx, 0);
     return SP_OK;
   };
   for (int i = 0; i < sp::binned_shape_count() && rc == SP_OK; ++i) {
@@ -1109,7 +1140,7 @@ int sp_merge(sp_ctx* ctx, const uint32_t* routers, uint32_t n, uint32_t dst_rout
   // LDCA, all of them in one pass: the sources keep theirs pending, and an
   // LDCA that is known to be zero is not read.  Without pending planes the
   // whole sketches are ORed by one plain pass.
-  bool pending = ctx->planes_dirty[dst_router];
+  bool pending = planes_pending(ctx, dst_router);
   std::vector<sp::FoldSrc> folds;
   folds.reserve(n + 1);
   if (pending) folds.push_back(sp::FoldSrc{ctx->planes[dst_router], nullptr, nullptr});
@@ -1117,10 +1148,10 @@ int sp_merge(sp_ctx* ctx, const uint32_t* routers, uint32_t n, uint32_t dst_rout
     const uint32_t r = routers[i];
     if (r == dst_router) continue;
     srcs.push_back(ctx->seav(r));
-    const bool dirty = ctx->planes_dirty[r];
+    const bool dirty = planes_pending(ctx, r);
     pending = pending || dirty;
     folds.push_back(sp::FoldSrc{dirty ? ctx->planes[r] : nullptr, ctx->ldca(r),
-                                ldca_known_zero(ctx, r) ? ctx->ovf + r : nullptr});
+                                spilled_if_zero(ctx, r)});
   }
   if (srcs.empty()) return fold_router(ctx, dst_router);
   if (ctx->captured && pending) {
@@ -1131,7 +1162,7 @@ int sp_merge(sp_ctx* ctx, const uint32_t* routers, uint32_t n, uint32_t dst_rout
     if (rc != SP_OK) return rc;
     pending = false;
   }
-  const uint32_t* fresh = ldca_known_zero(ctx, dst_router) ? ctx->ovf + dst_router : nullptr;
+  const uint32_t* fresh = spilled_if_zero(ctx, dst_router);
   ctx->ldca_zero[dst_router] = false;
   if (!pending)
     return sp::launch_merge(ctx->seav(dst_router), srcs.data(), (uint32_t)srcs.size(), ctx->stride, ctx->stream) ==
@@ -1349,8 +1380,9 @@ int sp_import(sp_ctx* ctx, uint32_t router, const void* host_buf, uint64_t n) {
       h.lc_log2 != ctx->p.lc_log2 || h.theta != ctx->p.theta || h.seed != ctx->p.seed ||
       h.seav_bytes != ctx->seav_bytes || h.ldca_bytes != ctx->ldca_bytes)
     return SP_ERR_CHECKSUM;
-  ctx->planes_dirty[router] = false;
+  ctx->planes_dirty[router] = false;               // pending planes go with the sketch they belong to
   ctx->ldca_zero[router] = false;
+  if (cudaMemsetAsync(ctx->flags + router, 0, sizeof(sp::RouterFlags), ctx->stream) != cudaSuccess) return SP_ERR_CUDA;
   if (cudaMemcpyAsync(ctx->seav(router), in + sizeof(h), ctx->seav_bytes, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
       cudaMemcpyAsync(ctx->ldca(router), in + sizeof(h) + ctx->seav_bytes, ctx->ldca_bytes, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess)
     return SP_ERR_CUDA;

@@ -81,6 +81,17 @@ struct BinShape {
 int binned_shape_count();
 BinShape binned_shape(int i);   // i in [0, binned_shape_count()); 0 is the default
 
+// What the device keeps of a router; its zeroing clears both.
+//   spilled: a pair's LDCA bit bypassed the lists.
+//   pending: the planes hold bits of the present window.  Set by a round's first
+//     k_bin; cleared with the LDCA (zeroing, import, the close of a slice) and, in
+//     a context with recorded calls, by a fold.  The launches of such a context
+//     go by it, since a replay finds other planes than the capture did; without
+//     recorded calls the host knows as much and passes plain arguments.
+struct RouterFlags {
+  uint32_t spilled, pending;
+};
+
 // Scratch of the binned scan (sp_scan_binned.cu), shared by a context's routers.
 struct BinnedScratch {
   uint32_t* lists = nullptr;    // [kBinRows][ctas][cap] hips; a plane's lists are consecutive
@@ -93,21 +104,23 @@ struct BinnedScratch {
   uint64_t list_words = 0;      // hips the lists allocation holds
   uint64_t max_pairs = 0;       // pairs per binning round the lists are sized for
   int fold_grid = 0;
-  uint32_t* ovf = nullptr;      // the router's flag: set when a pair's LDCA bit bypassed the lists
+  RouterFlags* flags = nullptr; // the router's
+  uint32_t* prior = nullptr;    // in a context with recorded calls, a device word: the router's `pending` before
+                                // the round's k_bin, which k_apply takes instead of `accumulate`
 };
 
 // ---- launchers (return cudaGetLastError() of the launch) -------------------
 cudaError_t launch_zero(void* dev, uint64_t bytes, cudaStream_t s);
-// launch_zero, and flags[0, n_flags) = 0 in the same launch
-cudaError_t launch_zero_flags(void* dev, uint64_t bytes, uint32_t* flags, uint32_t n_flags, cudaStream_t s);
+// launch_zero, and the flags of n routers in the same launch
+cudaError_t launch_zero_flags(void* dev, uint64_t bytes, RouterFlags* flags, uint32_t n, cudaStream_t s);
 // A set of a context's routers (at most 4,096), as a kernel argument.
 struct RouterSet {
   uint32_t w[128];
 };
 // Zeroes routers first .. first + count - 1 (sketches of `stride` bytes from
-// base) and their flags ovf; the LDCA of a router in `clean` only if its flag is set.
+// base) and their flags; the LDCA of a router in `clean` only if it has spilled.
 cudaError_t launch_reset(uint8_t* base, uint64_t stride, uint64_t seav_pad, uint32_t first, uint32_t count,
-                         const RouterSet& clean, uint32_t* ovf, cudaStream_t s);
+                         const RouterSet& clean, RouterFlags* flags, cudaStream_t s);
 cudaError_t launch_scan(const DevParams& d, uint8_t* seav, uint32_t* ldca,
                         const uint32_t* pairs, uint64_t n_pairs, int grid, cudaStream_t s);
 int scan_grid(const DevParams& d);
@@ -141,17 +154,17 @@ cudaError_t launch_scan_binned(const DevParams& d, uint8_t* seav, uint32_t* ldca
 // and nothing but binned rounds wrote it since; the fold then writes the
 // transposed planes without reading the LDCA, unless the flag is set.
 // nullptr: ldca |= transpose(planes).
+// pending: a device word, no fold when it is 0 (nullptr: always).
 cudaError_t launch_fold(const DevParams& d, const uint32_t* planes, uint32_t* ldca, int grid, cudaStream_t st,
-                        const uint32_t* fresh = nullptr);
+                        const uint32_t* fresh, const uint32_t* pending);
 // Up to kFoldMaxSrc routers folded into one LDCA: a router's pending planes
-// (null: none) and its LDCA, read unless null, or unless ovf is not null and
-// the flag it points at is 0 (the LDCA is still all zero then, see
-// BinnedScratch::ovf).
+// (null: none) and its LDCA, read unless null, or unless spilled is not null and
+// the word it points at is 0 (the LDCA is still all zero then).
 constexpr int kFoldMaxSrc = 32;
 struct FoldSrc {
   const uint32_t* planes;
   const uint32_t* ldca;
-  const uint32_t* ovf;
+  const uint32_t* spilled;
 };
 struct FoldSrcs {
   FoldSrc s[kFoldMaxSrc];
@@ -159,7 +172,7 @@ struct FoldSrcs {
 };
 // ldca |= transpose(OR of the sources' planes) | OR of their LDCAs; fresh as in launch_fold
 cudaError_t launch_fold_multi(const DevParams& d, const FoldSrcs& src, uint32_t* ldca, int grid, cudaStream_t st,
-                              const uint32_t* fresh);
+                              const uint32_t* fresh, const uint32_t* pending = nullptr);
 // Sliding window stamps (Sec. 5.2): one byte per bit holding the id of the
 // last slice that set it, id(t) = t mod 255 + 1 (0 = never set).  Byte j of
 // active_mask4 is 0xFF iff byte j of s is an active stamp: non-zero, of age
@@ -190,11 +203,12 @@ __device__ __forceinline__ uint32_t active32(const uint4& a, const uint4& b, uin
 // router's slice counter t in device memory (slice id t mod 255 + 1)
 // stamps id(t) on the counters of the slice sketch's set bits, then clears the sketch
 cudaError_t launch_commit(uint32_t* seav, uint8_t* st_seav, uint64_t seav_words, uint32_t* ldca,
-                          uint8_t* st_ldca, uint64_t ldca_words, const uint64_t* clock, cudaStream_t s);
+                          uint8_t* st_ldca, uint64_t ldca_words, const uint64_t* clock, uint32_t* pending,
+                          cudaStream_t s);
 // launch_commit, and the window's bits (active stamps) into wseav / wldca
 cudaError_t launch_commit_window(uint32_t* seav, uint8_t* st_seav, uint64_t seav_words, uint32_t* ldca,
                                  uint8_t* st_ldca, uint64_t ldca_words, uint32_t* wseav, uint32_t* wldca,
-                                 const uint64_t* clock, uint32_t k, cudaStream_t s);
+                                 const uint64_t* clock, uint32_t k, uint32_t* pending, cudaStream_t s);
 // t += 1, then the sweep of segment (t mod (255 - k)) of the router's stamps[0, bytes)
 cudaError_t launch_tick_clean(uint8_t* stamps, uint64_t bytes, uint64_t* clock, uint32_t k, cudaStream_t s);
 cudaError_t launch_merge_stamp(uint8_t* dst, const uint8_t* const* srcs, uint32_t n_src, uint64_t bytes,

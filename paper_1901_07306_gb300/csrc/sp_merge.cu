@@ -23,23 +23,23 @@ struct SrcList {
 };
 
 __global__ void __launch_bounds__(kThreads)
-k_zero(uint4* __restrict__ p, uint64_t n16, uint32_t* __restrict__ flags, uint32_t n_flags) {
+k_zero(uint4* __restrict__ p, uint64_t n16, RouterFlags* __restrict__ flags, uint32_t n) {
   const uint4 z = make_uint4(0u, 0u, 0u, 0u);
   const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (uint64_t i = gid; i < n16; i += (uint64_t)gridDim.x * blockDim.x) p[i] = z;
-  for (uint64_t i = gid; i < n_flags; i += (uint64_t)gridDim.x * blockDim.x) flags[i] = 0u;
+  for (uint64_t i = gid; i < n; i += (uint64_t)gridDim.x * blockDim.x) flags[i] = RouterFlags{0u, 0u};
 }
 
 // Routers first .. first + count - 1 of a context: the SEAV, and the LDCA
-// unless bit r of `clean` is set and ovf[r] is 0.  Every block takes its share
+// unless bit r of `clean` is set and the router has not spilled.  Every block takes its share
 // of every router (one that is zeroed whole among many skipped ones is spread
 // over the chip).  Blocks read all flags, so the caller clears them after the launch.
 __global__ void __launch_bounds__(kThreads)
 k_reset(uint8_t* __restrict__ base, uint64_t stride, uint64_t seav16, uint32_t first, uint32_t count,
-        RouterSet clean, const uint32_t* __restrict__ ovf) {
+        RouterSet clean, const RouterFlags* __restrict__ flags) {
   const uint4 z = make_uint4(0u, 0u, 0u, 0u);
   for (uint32_t r = first; r < first + count; ++r) {
-    const bool skip = ((clean.w[r >> 5] >> (r & 31u)) & 1u) != 0u && ovf[r] == 0u;
+    const bool skip = ((clean.w[r >> 5] >> (r & 31u)) & 1u) != 0u && flags[r].spilled == 0u;
     uint4* p = reinterpret_cast<uint4*>(base + (uint64_t)r * stride);
     const uint64_t n16 = skip ? seav16 : stride / 16;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (uint64_t)gridDim.x * blockDim.x)
@@ -70,13 +70,13 @@ int stream_grid() {
 
 // bytes must be a multiple of 16 and the pointer 16-byte aligned (sketch
 // regions are padded to 256 bytes by the context).
-cudaError_t launch_zero_flags(void* dev, uint64_t bytes, uint32_t* flags, uint32_t n_flags, cudaStream_t s) {
+cudaError_t launch_zero_flags(void* dev, uint64_t bytes, RouterFlags* flags, uint32_t n, cudaStream_t s) {
   const uint64_t n16 = bytes / 16;
-  const uint64_t work = n16 > n_flags ? n16 : n_flags;
+  const uint64_t work = n16 > n ? n16 : n;
   if (work == 0) return cudaSuccess;
   uint64_t grid = (work + kThreads - 1) / kThreads;
   if (grid > (uint64_t)stream_grid()) grid = stream_grid();
-  k_zero<<<(unsigned)grid, kThreads, 0, s>>>(reinterpret_cast<uint4*>(dev), n16, flags, n_flags);
+  k_zero<<<(unsigned)grid, kThreads, 0, s>>>(reinterpret_cast<uint4*>(dev), n16, flags, n);
   return cudaGetLastError();
 }
 
@@ -85,13 +85,13 @@ cudaError_t launch_zero(void* dev, uint64_t bytes, cudaStream_t s) {
 }
 
 cudaError_t launch_reset(uint8_t* base, uint64_t stride, uint64_t seav_pad, uint32_t first, uint32_t count,
-                         const RouterSet& clean, uint32_t* ovf, cudaStream_t s) {
+                         const RouterSet& clean, RouterFlags* flags, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
   uint64_t grid = (stride / 16 + kThreads - 1) / kThreads;
   if (grid > (uint64_t)stream_grid()) grid = stream_grid();
-  k_reset<<<(unsigned)grid, kThreads, 0, s>>>(base, stride, seav_pad / 16, first, count, clean, ovf);
+  k_reset<<<(unsigned)grid, kThreads, 0, s>>>(base, stride, seav_pad / 16, first, count, clean, flags);
   const cudaError_t e = cudaGetLastError();
-  return e != cudaSuccess ? e : cudaMemsetAsync(ovf + first, 0, sizeof(uint32_t) * count, s);
+  return e != cudaSuccess ? e : cudaMemsetAsync(flags + first, 0, sizeof(RouterFlags) * count, s);
 }
 
 cudaError_t launch_merge(uint8_t* dst, const uint8_t* const* srcs, uint32_t n_src,

@@ -113,7 +113,7 @@ template <int THREADS, int STAGE, int TPR, int PER_SM>
 __global__ void __launch_bounds__(THREADS, PER_SM)
 k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
       BinSrc src, uint32_t* __restrict__ lists, uint32_t* __restrict__ counts, uint32_t cap,
-      bool append, uint32_t rot, uint32_t* __restrict__ ovf) {
+      bool append, uint32_t rot, RouterFlags* __restrict__ flags, uint32_t* __restrict__ prior) {
   constexpr int QUADS = THREADS * kVec;               // 16-byte loads of a whole tile
   constexpr int TILE = QUADS * 2;
   constexpr int QUEUE = TPR * TILE / 32;              // sampled pairs per round: 4x the expected 2^-7
@@ -140,7 +140,7 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
   // the router's flag tells the fold that the LDCA is no longer all zero
   auto spill = [&](uint32_t hip, uint32_t b) {     // b: the row
     ldca_red(d, ldca, hip, b >> row_shift);
-    if (ovf) *ovf = 1u;
+    flags->spilled = 1u;
   };
   // A stream is a body of 16-byte quads (two pairs) and up to two single
   // pairs: its first one when it starts 8 bytes off a 16-byte boundary, its last
@@ -173,6 +173,10 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
     for (int e = 0; e < kBinMaxSrc / 32; ++e) pref[lane * (kBinMaxSrc / 32) + (uint32_t)e + 1] = incl - acc + sum[e];
     if (lane == 0) pref[0] = 0;
     if (tid == 0) s_qn[0] = s_qn[1] = s_on[0] = s_on[1] = 0;
+    if (tid == 0 && cta == 0 && !append) {         // the round's first launch: its k_apply makes the planes pending
+      if (prior != nullptr) *prior = flags->pending;
+      flags->pending = 1u;
+    }
   }
   auto list_of = [&](uint32_t b) { return lists + ((uint64_t)b * G + cta) * cap; };
   for (uint32_t b = tid; b < bins; b += THREADS) {
@@ -434,7 +438,7 @@ template <int LR, int THREADS, int LCL, int SPLIT>
 __global__ void __launch_bounds__(THREADS, 1536 / THREADS)
 k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restrict__ counts,
         uint32_t G, uint32_t cap, const uint32_t* planes, const __grid_constant__ CUtensorMap map, uint32_t box,
-        bool accumulate) {
+        bool accumulate, const uint32_t* prior) {
   extern __shared__ __align__(128) uint32_t s_plane[];
   constexpr int LRP = LR / SPLIT;                                  // rows of this block
   constexpr uint32_t NG = THREADS / 8;
@@ -478,6 +482,7 @@ k_apply(DevParams d, const uint32_t* __restrict__ lists, const uint32_t* __restr
     bw[r] = d.hb[2 + row0 + r];
   }
   for (uint32_t i = tid; i < G; i += THREADS) s_count[i] = counts[i];
+  if (prior != nullptr) accumulate = *prior != 0u;
   for (uint32_t u = tid; u < chunks * 2u; u += THREADS)             // 16-byte units, consecutive lanes
     *reinterpret_cast<uint4*>(s_plane + u * 4u) =
         accumulate ? *reinterpret_cast<const uint4*>(src + (u >> 1) * chunk_stride + (u & 1u) * 4u)
@@ -616,7 +621,7 @@ __device__ __forceinline__ void transpose8x4(uint32_t (&x)[8], uint32_t lane) {
 // A source's LDCA is read unless it is null or a flag beside it says that it is
 // still all zero (FoldSrc).
 __device__ __forceinline__ const uint32_t* live_ldca(const FoldSrc& s) {
-  return (s.ldca == nullptr || (s.ovf != nullptr && *s.ovf == 0u)) ? nullptr : s.ldca;
+  return (s.ldca == nullptr || (s.spilled != nullptr && *s.spilled == 0u)) ? nullptr : s.ldca;
 }
 
 // k < 256.  A warp task is 8 consecutive plane words J0 .. J0 + 7 (one 32-byte
@@ -624,7 +629,9 @@ __device__ __forceinline__ const uint32_t* live_ldca(const FoldSrc& s) {
 // memory) times 4 consecutive LDC words: it transposes 32 planes x 32 LDCs per
 // word and ORs the result into the lanes' LDC lines.
 __global__ void __launch_bounds__(256, 2)
-k_fold(FoldSrcs src, uint32_t* ldca, uint32_t W, uint32_t k_log2, const uint32_t* __restrict__ fresh) {
+k_fold(FoldSrcs src, uint32_t* ldca, uint32_t W, uint32_t k_log2, const uint32_t* __restrict__ fresh,
+       const uint32_t* __restrict__ pending) {
+  if (pending != nullptr && *pending == 0u) return;
   const bool write_only = fresh != nullptr && *fresh == 0u;       // the LDCA is all zero: no read
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t wpl = 1u << (k_log2 - 5u);                       // words per LDC
@@ -687,7 +694,9 @@ k_fold(FoldSrcs src, uint32_t* ldca, uint32_t W, uint32_t k_log2, const uint32_t
 constexpr int kFold8Threads = 128;
 template <bool kMulti>
 __global__ void __launch_bounds__(kFold8Threads, kMulti ? 3 : 4)
-k_fold8(FoldSrcs src, uint32_t* ldca, uint32_t W, uint32_t k_log2, const uint32_t* __restrict__ fresh) {
+k_fold8(FoldSrcs src, uint32_t* ldca, uint32_t W, uint32_t k_log2, const uint32_t* __restrict__ fresh,
+        const uint32_t* __restrict__ pending) {
+  if (pending != nullptr && *pending == 0u) return;
   const bool write_only = fresh != nullptr && *fresh == 0u;       // the LDCA is all zero: no read
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t wpl = 1u << (k_log2 - 5u);                       // words per LDC, >= 8
@@ -762,7 +771,8 @@ cudaError_t bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, const B
   auto kern = k_bin<THREADS, STAGE, TPR, PER_SM>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bin_smem);
   if (e != cudaSuccess) return e;
-  kern<<<s.ctas, THREADS, bin_smem, st>>>(d, seav, ldca, src, s.lists, s.counts, cap, append, rot, s.ovf);
+  kern<<<s.ctas, THREADS, bin_smem, st>>>(d, seav, ldca, src, s.lists, s.counts, cap, append, rot, s.flags,
+                                           s.prior);
   return cudaGetLastError();
 }
 
@@ -804,7 +814,8 @@ cudaError_t apply_round_t(const DevParams& d, const BinnedScratch& s, uint32_t c
   while (chunks % box != 0u) --box;
   CUtensorMap map;
   if ((e = plane_map(s.planes, bins, chunks * (uint32_t)SPLIT, box, &map)) != cudaSuccess) return e;
-  kern<<<bins * SPLIT, THREADS, apply_smem, st>>>(d, s.lists, s.counts, n_lists, cap, s.planes, map, box, accumulate);
+  kern<<<bins * SPLIT, THREADS, apply_smem, st>>>(d, s.lists, s.counts, n_lists, cap, s.planes, map, box, accumulate,
+                                             s.prior);
   return cudaGetLastError();
 }
 
@@ -872,21 +883,21 @@ int binned_ctas(const BinShape& shape) { return sm_count() * (int)shape.per_sm; 
 int binned_fold_grid() { return sm_count() * 8; }
 
 cudaError_t launch_fold_multi(const DevParams& d, const FoldSrcs& src, uint32_t* ldca, int grid, cudaStream_t st,
-                              const uint32_t* fresh) {
+                              const uint32_t* fresh, const uint32_t* pending) {
   const uint32_t words = (uint32_t)(((uint64_t)d.lr << d.lc_log2) >> 5);
-  if (d.k_log2 < 8) k_fold<<<grid, 256, 0, st>>>(src, ldca, words, d.k_log2, fresh);
+  if (d.k_log2 < 8) k_fold<<<grid, 256, 0, st>>>(src, ldca, words, d.k_log2, fresh, pending);
   else if (src.count == 1 && src.s[0].planes && !src.s[0].ldca)
-    k_fold8<false><<<2 * grid, kFold8Threads, 0, st>>>(src, ldca, words, d.k_log2, fresh);
-  else k_fold8<true><<<2 * grid, kFold8Threads, 0, st>>>(src, ldca, words, d.k_log2, fresh);
+    k_fold8<false><<<2 * grid, kFold8Threads, 0, st>>>(src, ldca, words, d.k_log2, fresh, pending);
+  else k_fold8<true><<<2 * grid, kFold8Threads, 0, st>>>(src, ldca, words, d.k_log2, fresh, pending);
   return cudaGetLastError();
 }
 
 cudaError_t launch_fold(const DevParams& d, const uint32_t* planes, uint32_t* ldca, int grid, cudaStream_t st,
-                        const uint32_t* fresh) {
+                        const uint32_t* fresh, const uint32_t* pending) {
   FoldSrcs src{};
   src.s[0].planes = planes;
   src.count = 1;
-  return launch_fold_multi(d, src, ldca, grid, st, fresh);
+  return launch_fold_multi(d, src, ldca, grid, st, fresh, pending);
 }
 
 BinSrc bin_src_one(const uint32_t* pairs, uint64_t n_pairs) {

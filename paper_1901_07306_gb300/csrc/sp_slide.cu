@@ -95,11 +95,13 @@ __device__ __forceinline__ void store8(uint4* st, uint64_t i, const uint32_t (&v
 // Commit of one slice: every bit set in the slice's bit sketch stamps its
 // counter with the slice id; counters of unset bits keep their stamp.  The
 // slice sketch is consumed (nonzero words cleared), so the next updates of the
-// router start a fresh slice sketch.  Zero words cost one 4-byte read.
+// router start a fresh slice sketch.  Zero words cost one 4-byte read.  What
+// the planes hold belongs to the slices before then: *pending = 0.
 __global__ void __launch_bounds__(kThreads)
 k_commit(uint32_t* __restrict__ seav, uint4* __restrict__ st_seav, uint64_t seav_words,
          uint32_t* __restrict__ ldca, uint4* __restrict__ st_ldca, uint64_t ldca_words,
-         const uint64_t* __restrict__ clock) {
+         const uint64_t* __restrict__ clock, uint32_t* __restrict__ pending) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *pending = 0u;
   const uint32_t id4 = slice_id(clock) * 0x01010101u;
   const uint64_t n = seav_words + ldca_words;
   for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x) {
@@ -125,7 +127,8 @@ __global__ void __launch_bounds__(kThreads)
 k_commit_window(uint32_t* __restrict__ seav, uint4* __restrict__ st_seav, uint64_t seav_words,
                 uint32_t* __restrict__ ldca, uint4* __restrict__ st_ldca, uint64_t ldca_words,
                 uint32_t* __restrict__ wseav, uint32_t* __restrict__ wldca, const uint64_t* __restrict__ clock,
-                uint32_t k) {
+                uint32_t k, uint32_t* __restrict__ pending) {
+  if (ldca_words != 0u && blockIdx.x == 0 && threadIdx.x == 0) *pending = 0u;
   const uint32_t id4 = slice_id(clock) * 0x01010101u, k4 = k * 0x01010101u;   // k <= 128 < 256
   const uint64_t n = seav_words + ldca_words;
   for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (uint64_t)gridDim.x * blockDim.x) {
@@ -205,19 +208,19 @@ unsigned grid_for(uint64_t work) {
 }  // namespace
 
 cudaError_t launch_commit(uint32_t* seav, uint8_t* st_seav, uint64_t seav_words, uint32_t* ldca,
-                          uint8_t* st_ldca, uint64_t ldca_words, const uint64_t* clock, cudaStream_t s) {
+                          uint8_t* st_ldca, uint64_t ldca_words, const uint64_t* clock, uint32_t* pending, cudaStream_t s) {
   k_commit<<<grid_for(seav_words + ldca_words), kThreads, 0, s>>>(
       seav, reinterpret_cast<uint4*>(st_seav), seav_words, ldca, reinterpret_cast<uint4*>(st_ldca), ldca_words,
-      clock);
+      clock, pending);
   return cudaGetLastError();
 }
 
 cudaError_t launch_commit_window(uint32_t* seav, uint8_t* st_seav, uint64_t seav_words, uint32_t* ldca,
                                  uint8_t* st_ldca, uint64_t ldca_words, uint32_t* wseav, uint32_t* wldca,
-                                 const uint64_t* clock, uint32_t k, cudaStream_t s) {
+                                 const uint64_t* clock, uint32_t k, uint32_t* pending, cudaStream_t s) {
   k_commit_window<<<grid_for(seav_words + ldca_words), kThreads, 0, s>>>(
       seav, reinterpret_cast<uint4*>(st_seav), seav_words, ldca, reinterpret_cast<uint4*>(st_ldca), ldca_words,
-      wseav, wldca, clock, k);
+      wseav, wldca, clock, k, pending);
   return cudaGetLastError();
 }
 
