@@ -181,7 +181,11 @@ SP_API int sp_create(const sp_params* p, void* cuda_stream, sp_ctx** out);
 SP_API void sp_destroy(sp_ctx* ctx);
 
 /* Replaces the context's stream (work already issued stays ordered on the old
- * one; the caller synchronises if needed). */
+ * one; the caller synchronises if needed).  Updates in the direct form and
+ * batched scans need nothing: bits may be set in any order and at the same
+ * time, and the batched scans of two streams follow one another where they
+ * share scratch memory.  Binned updates share the context's lists and detects
+ * its result buffers: those are ordered by the caller. */
 SP_API int sp_set_stream(sp_ctx* ctx, void* cuda_stream);
 
 /* Bound of every wait of the context on its stream (sp_results, sp_detect,

@@ -158,6 +158,10 @@ struct sp_ctx {
   static constexpr int kTableRing = 4;
   TableSlot tables[kTableRing];
   uint32_t table_next = 0;
+  // Table scans that draw tickets run one at a time: ev_table marks the last
+  // one, and the first on another stream waits for it there.
+  cudaEvent_t ev_table = nullptr;
+  bool table_elsewhere = false;             // the stream was replaced since that scan
   int multi_threads = 256;
   int multi_grid = 0;
   uint32_t bs_shape_index = 0;              // staging shape of the binned scan (sp_autotune_binned)
@@ -379,6 +383,7 @@ void sp_destroy(sp_ctx* ctx) {
   cudaFree(ctx->est_table);
   if (ctx->ev_wait) cudaEventDestroy(ctx->ev_wait);
   if (ctx->ev_arena) cudaEventDestroy(ctx->ev_arena);
+  if (ctx->ev_table) cudaEventDestroy(ctx->ev_table);
   delete ctx;
 }
 
@@ -435,7 +440,9 @@ int sp_create(const sp_params* p, void* cuda_stream, sp_ctx** out) {
     cudaGetLastError();
     rc = SP_ERR_NOMEM;
   }
-  if (rc == SP_OK && cudaEventCreateWithFlags(&c->ev_wait, cudaEventDisableTiming) != cudaSuccess) rc = SP_ERR_CUDA;
+  if (rc == SP_OK && (cudaEventCreateWithFlags(&c->ev_wait, cudaEventDisableTiming) != cudaSuccess ||
+                      cudaEventCreateWithFlags(&c->ev_table, cudaEventDisableTiming) != cudaSuccess))
+    rc = SP_ERR_CUDA;
   if (rc == SP_OK) {
     const uint32_t k = 1u << p->k_log2;
     double* table = static_cast<double*>(malloc((k + 1) * sizeof(double)));
@@ -488,6 +495,7 @@ int sp_create(const sp_params* p, void* cuda_stream, sp_ctx** out) {
 int sp_set_stream(sp_ctx* ctx, void* cuda_stream) {
   if (!ctx) return SP_ERR_PARAM;
   ctx->stream = static_cast<cudaStream_t>(cuda_stream);
+  ctx->table_elsewhere = true;
   return SP_OK;
 }
 
@@ -839,7 +847,19 @@ static int grow_table_slot(sp_ctx* ctx, sp_ctx::TableSlot& t, uint32_t n) {
   return SP_OK;
 }
 
+// Puts the stream behind the last table scan when that one is on another
+// stream: it may still draw from the context's ticket and read a slot's table.
+// (An event that was never recorded is no wait.)
+static int order_table_scans(sp_ctx* ctx) {
+  if (!ctx->table_elsewhere) return SP_OK;
+  if (cudaStreamWaitEvent(ctx->stream, ctx->ev_table, 0) != cudaSuccess) return SP_ERR_CUDA;
+  ctx->table_elsewhere = false;
+  return SP_OK;
+}
+
 static int upload_table(sp_ctx* ctx, const sp_batch* tab, uint32_t n, const sp_batch** dev) {
+  const int orc = order_table_scans(ctx);
+  if (orc != SP_OK) return orc;
   sp_ctx::TableSlot& t = ctx->tables[ctx->table_next++ % sp_ctx::kTableRing];
   const int grc = grow_table_slot(ctx, t, n);
   if (grc != SP_OK) return grc;
@@ -857,13 +877,18 @@ static int upload_table(sp_ctx* ctx, const sp_batch* tab, uint32_t n, const sp_b
 
 static int launch_table(sp_ctx* ctx, const sp_batch* dev_tab, uint32_t n) {
   constexpr uint32_t kMaxTable = 8192;
+  // a recorded launch may run beside any other one: no ticket
+  const bool recorded = capturing(ctx->stream);
+  const int rc = recorded ? SP_OK : order_table_scans(ctx);
+  if (rc != SP_OK) return rc;
   for (uint32_t i = 0; i < n; i += kMaxTable) {
     const uint32_t m = (n - i) < kMaxTable ? (n - i) : kMaxTable;
     if (sp::launch_scan_multi(ctx->d, ctx->sketches, ctx->stride, ctx->seav_pad, ctx->p.n_routers, dev_tab + i, m,
-                              ctx->kerr(), ctx->ticket(), ctx->multi_threads, ctx->multi_grid, ctx->stream) != cudaSuccess)
+                              ctx->kerr(), recorded ? nullptr : ctx->ticket(), ctx->multi_threads, ctx->multi_grid,
+                              ctx->stream) != cudaSuccess)
       return SP_ERR_CUDA;
   }
-  return SP_OK;
+  return recorded || cudaEventRecord(ctx->ev_table, ctx->stream) == cudaSuccess ? SP_OK : SP_ERR_CUDA;
 }
 
 int sp_reserve(sp_ctx* ctx, uint32_t first, uint32_t count) {

@@ -196,10 +196,13 @@ int grid_for() {
 // the chunk before is scanned, and finds the chunk's batch by binary search.
 // Routers index the context's sketches.  Tickets keep the chunks in flight next
 // to each other in the table, whose batches the host groups by router: with
-// chunks block, block + grid, ... the blocks drifted apart until the REDs went to
-// more sketches than L2 holds and nearly each one missed (15 routers of profile
-// D x 2.7 M uniform pairs: 4,226 us, 1,662 with tickets).  A chunk draws one
+// chunks block, block + grid, ... the blocks drift apart until the REDs go to
+// more sketches than L2 holds and nearly each one misses (15 routers of profile
+// D x 2.7 M uniform pairs: 4,334 us, 1,748 with tickets).  A chunk draws one
 // ticket, so the drawer of the last one zeroes the counter for the next launch.
+// A counter serves one launch at a time: a launch that may run beside another
+// one (a recorded one, replayed at any time) gets none and takes chunks block,
+// block + grid, ..., which share nothing.
 constexpr uint32_t kChunk = 2048;
 
 template <int LR, int THREADS>
@@ -237,11 +240,11 @@ k_scan_multi(DevParams d, uint8_t* __restrict__ sketches, uint64_t stride, uint6
     if (tid == THREADS - 1) s_carry += s_tmp[tid];
     __syncthreads();
   }
-  const uint64_t total = s_pref[n_batches];               // < 2^32 chunks
+  const uint64_t total = s_pref[n_batches];               // < 2^32 chunks where tickets are drawn
   __shared__ uint32_t s_next[2];
-  uint32_t g = blockIdx.x;                                 // the first chunk; then gridDim.x + ticket
+  uint64_t g = blockIdx.x;                                 // the first chunk; then gridDim.x + ticket
   for (uint32_t turn = 0; g < total; turn ^= 1u) {
-    if (tid == 0) {
+    if (ticket != nullptr && tid == 0) {
       const uint32_t t = atomicAdd(ticket, 1u);            // one per chunk
       if (t == (uint32_t)total - 1u) *ticket = 0u;
       s_next[turn] = gridDim.x + t;
@@ -260,6 +263,10 @@ k_scan_multi(DevParams d, uint8_t* __restrict__ sketches, uint64_t stride, uint6
     for (uint32_t i = tid; i < cnt; i += THREADS) {
       const uint2 v = __ldcs(p2 + i);
       scan_pair<LR>(d, seav, ldca, v.x, v.y, tau_mask);
+    }
+    if (ticket == nullptr) {
+      g += gridDim.x;
+      continue;
     }
     __syncthreads();
     g = s_next[turn];
