@@ -876,13 +876,12 @@ static int upload_table(sp_ctx* ctx, const sp_batch* tab, uint32_t n, const sp_b
 }
 
 static int launch_table(sp_ctx* ctx, const sp_batch* dev_tab, uint32_t n) {
-  constexpr uint32_t kMaxTable = 8192;
   // a recorded launch may run beside any other one: no ticket
   const bool recorded = capturing(ctx->stream);
   const int rc = recorded ? SP_OK : order_table_scans(ctx);
   if (rc != SP_OK) return rc;
-  for (uint32_t i = 0; i < n; i += kMaxTable) {
-    const uint32_t m = (n - i) < kMaxTable ? (n - i) : kMaxTable;
+  for (uint32_t i = 0; i < n; i += sp::kMaxTable) {
+    const uint32_t m = (n - i) < sp::kMaxTable ? (n - i) : sp::kMaxTable;
     if (sp::launch_scan_multi(ctx->d, ctx->sketches, ctx->stride, ctx->seav_pad, ctx->p.n_routers, dev_tab + i, m,
                               ctx->kerr(), recorded ? nullptr : ctx->ticket(), ctx->multi_threads, ctx->multi_grid,
                               ctx->stream) != cudaSuccess)
@@ -1016,7 +1015,7 @@ int sp_update_batched_host(sp_ctx* ctx, uint32_t n_batches, const uint32_t* rout
 int sp_update_batched_device(sp_ctx* ctx, const sp_batch* dev_batches, uint32_t n_batches) {
   if (!ctx) return SP_ERR_PARAM;
   if (n_batches == 0) return SP_OK;
-  if (!dev_batches || n_batches > 8192) return SP_ERR_PARAM;
+  if (!dev_batches || n_batches > sp::kMaxTable) return SP_ERR_PARAM;
   note_capture(ctx);
   // the table is read on the device: any router may receive bits
   for (uint32_t r = 0; r < ctx->p.n_routers; ++r) {

@@ -124,7 +124,9 @@ cudaError_t launch_reset(uint8_t* base, uint64_t stride, uint64_t seav_pad, uint
 cudaError_t launch_scan(const DevParams& d, uint8_t* seav, uint32_t* ldca,
                         const uint32_t* pairs, uint64_t n_pairs, int grid, cudaStream_t s);
 int scan_grid(const DevParams& d);
-// batched direct scan over a device table of batches (sp_batch, include/superpoint.h);
+constexpr uint32_t kMaxTable = 8192;
+// batched direct scan over a device table of at most kMaxTable batches (sp_batch,
+// include/superpoint.h);
 // ticket: a device word, zero before the launch and after it, that no other
 // launch uses meanwhile; nullptr: the launch shares nothing with others
 cudaError_t launch_scan_multi(const DevParams& d, uint8_t* sketches, uint64_t stride, uint64_t seav_pad,

@@ -278,17 +278,19 @@ cudaError_t multi_lr(const DevParams& d, uint8_t* sketches, uint64_t stride, uin
                      const sp_batch* desc, uint32_t n_batches, uint32_t* err, uint32_t* ticket, int threads, int grid,
                      cudaStream_t s) {
   const size_t smem = ((size_t)n_batches + 1) * sizeof(uint64_t);
+  // the same limit from every call: none lowers it under another thread's launch
+  constexpr int kMost = (int)((kMaxTable + 1) * sizeof(uint64_t));
   switch (threads) {
     case 128:
-      cudaFuncSetAttribute(k_scan_multi<LR, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_scan_multi<LR, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
       k_scan_multi<LR, 128><<<grid, 128, smem, s>>>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket);
       break;
     case 512:
-      cudaFuncSetAttribute(k_scan_multi<LR, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_scan_multi<LR, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
       k_scan_multi<LR, 512><<<grid, 512, smem, s>>>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket);
       break;
     default:
-      cudaFuncSetAttribute(k_scan_multi<LR, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k_scan_multi<LR, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
       k_scan_multi<LR, 256><<<grid, 256, smem, s>>>(d, sketches, stride, seav_pad, n_routers, desc, n_batches, err, ticket);
       break;
   }

@@ -776,6 +776,13 @@ cudaError_t bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, const B
   return cudaGetLastError();
 }
 
+int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
 // The accumulator as a tensor [chunks][bins][8] of words; copies take `box`
 // chunks of one plane.
 cudaError_t plane_map(uint32_t* planes, uint32_t bins, uint32_t chunks, uint32_t box, CUtensorMap* map) {
@@ -800,6 +807,13 @@ cudaError_t plane_map(uint32_t* planes, uint32_t bins, uint32_t chunks, uint32_t
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// Dynamic shared memory of the largest k_apply: a plane of 2^20 bits, and the
+// counts of k = 32's lists with the most binning blocks (167 KiB in all on 152
+// SMs).  Every call sets the same limit, so that none lowers it under another
+// thread's launch of the same kernel (what a launch needs follows k, LC and the
+// staging shape).
+int apply_smem_most() { return (1 << 17) + 2 * sm_count() * (int)sizeof(uint32_t) * (1 << (kBinRowsLog2 - 5u)); }
+
 template <int LR, int THREADS, int LCL, int SPLIT = 1>
 cudaError_t apply_round_t(const DevParams& d, const BinnedScratch& s, uint32_t cap, bool accumulate, cudaStream_t st) {
   const uint32_t bins = 1u << d.k_log2;
@@ -807,7 +821,7 @@ cudaError_t apply_round_t(const DevParams& d, const BinnedScratch& s, uint32_t c
   const uint32_t n_lists = s.ctas << (kBinRowsLog2 - d.k_log2);                    // of a plane
   const size_t apply_smem = ((size_t)chunks * 8u + n_lists) * sizeof(uint32_t);    // the rows, the lists' counts
   auto kern = k_apply<LR, THREADS, LCL, SPLIT>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, apply_smem_most());
   if (e != cudaSuccess) return e;
   // chunks of a copy: a block's chunks in equal boxes of at most 256
   uint32_t box = chunks < 256u ? chunks : 256u;
@@ -869,13 +883,6 @@ uint32_t binned_list_cap(uint64_t n_pairs, const BinShape& shape, uint32_t ctas,
   uint64_t cap = (uint64_t)(m + 8.0 * sqrt(m + 1.0) + 32.0);
   cap = (cap + 7) & ~7ull;                                   // 32-byte list starts
   return (uint32_t)cap;
-}
-
-static int sm_count() {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
 }
 
 int binned_ctas(const BinShape& shape) { return sm_count() * (int)shape.per_sm; }
