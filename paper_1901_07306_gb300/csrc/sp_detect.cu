@@ -10,10 +10,10 @@
 //      its SEs falls below weight 3 -- AND only clears bits, so the pruning
 //      loses nothing against testing complete tuples (Sec. 3.2, SEU test).
 //   3. A complete tuple fixes every LP bit (Eq. 3, coverage constraint);
-//      ip = LP << r | RP goes to a per-warp queue.  Once enough are queued, or
-//      the warp has no SEA left, it tests the queued hosts together: the LDC union (AND over the LR
-//      rows, Sec. 3.3) of one host is read as LR lines of k bits spread over
-//      the lanes (one coalesced load per row and lane), z0 = k - popc by a
+//      ip = LP << r | RP goes to a per-warp queue.  Once enough are queued after
+//      a turn of 32 pairs, or the warp has no SEA left, it tests the queued hosts
+//      together: the LDC union (AND over the LR rows, Sec. 3.3) of one host is
+//      read as LR lines of k bits spread over the lanes (one coalesced load per row and lane), z0 = k - popc by a
 //      warp reduction.  The host survives when z0 <= Z_theta, the integer
 //      form of Est >= threshold (Eq. 4).  A full queue falls back to the
 //      same test in one lane.  For a sliding router (Sec. 5.2) a line word
@@ -105,6 +105,19 @@ template <bool kSliding>
 __device__ __forceinline__ uint32_t ldc_zeros(const DevParams& d, const LdcaRead& a, uint32_t ip) {
   const uint32_t wpl = 1u << (d.k_log2 - 5u);
   uint32_t ones = 0;
+  if (!kSliding && wpl >= 4u) {
+#pragma unroll 1
+    for (uint32_t w = 0; w < wpl; w += 4) {
+      uint4 u = make_uint4(kFull, kFull, kFull, kFull);
+#pragma unroll 1
+      for (uint32_t i = 0; i < d.lr; ++i) {
+        const uint4 v = *reinterpret_cast<const uint4*>(a.bits + ldc_line(d, ip, i) + w);
+        u.x &= v.x; u.y &= v.y; u.z &= v.z; u.w &= v.w;
+      }
+      ones += __popc(u.x) + __popc(u.y) + __popc(u.z) + __popc(u.w);
+    }
+    return (1u << d.k_log2) - ones;
+  }
 #pragma unroll 1
   for (uint32_t w = 0; w < wpl; ++w) {
     uint32_t u = kFull;
@@ -286,6 +299,26 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
   if (kStaged) stage_sea(rp, 0u);
   uint32_t join_local = 0;
   bool stop = false;
+  // The pairs of HSE(0) x HSE(1) in turns of one per lane (body: a lane's join
+  // from its pair on).  A turn that leaves kTestAt hosts queued is followed by
+  // their test, so that an SEA with hundreds of tuples does not fill the queue:
+  // a host that finds it full is tested in one lane, 32 round trips at k = 1,024
+  // (profile S, five hosts an SEA: 742 us with the test after each SEA, 248 so;
+  // ten an SEA 4,849 and 887).
+  auto join_turns = [&](uint32_t total, auto body) {
+    for (uint32_t first = 0; first < total && !stop; first += 32u) {
+      if (first + lane < total) body(first + lane);
+      __syncwarp();
+      const uint32_t nq = __shfl_sync(kFull, lane == 0 ? *queue_n : 0u, 0);   // one value for all lanes
+      if (nq >= kTestAt) {
+        test_queue<kSliding>(d, ldca, queue, min(nq, (uint32_t)kHostQueue), z_theta, f, pend, lane);
+        __syncwarp();
+        if (lane == 0) *queue_n = 0;
+        __syncwarp();
+      }
+      stop = __any_sync(kFull, stop);
+    }
+  };
   while (rp < n_sea && !stop) {
     // the join-bound flag (warp-uniform: lane 0 reads it, every lane sees its
     // value) is read here and tested after this SEA, so the read overlaps the
@@ -342,12 +375,12 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
         constexpr uint32_t kLp = 0x00FFFFFFu;
         const uint32_t total = n0 * n1;                            // <= 2^14: the float quotient is exact
         const float inv1 = 1.0f / (float)n1;
-        for (uint32_t t = lane; t < total && !stop; t += 32) {
+        join_turns(total, [&](uint32_t t) {
           const uint32_t t0 = (uint32_t)(((float)t + 0.5f) * inv1);
           const uint32_t e0 = entries[t0], e1 = entries[128u + t - t0 * n1];
-          if (((e0 ^ e1) & shared1) != 0u) continue;
+          if (((e0 ^ e1) & shared1) != 0u) return;
           const uint32_t p = ((e0 | e1) & kLp) | (e0 & e1 & ~kLp);
-          if (__popc(p >> 24) < 3) continue;
+          if (__popc(p >> 24) < 3) return;
           for (uint32_t i = 0; i < n2 && !stop; ++i) {
             const uint32_t e2 = entries[256u + i];
             const uint32_t q = ((p | e2) & kLp) | (p & e2 & ~kLp);
@@ -358,7 +391,7 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
               if (!emit_lp<kSliding>(d, ldca, rp, (q | e3) & kLp, z_theta, f, join_local, queue, queue_n)) stop = true;
             }
           }
-        }
+        });
       }
     } else {
       // 1. hot SEs per row
@@ -403,7 +436,7 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
         const uint32_t n1 = d.sr > 1 ? cnt[1] : 1u;
         const uint32_t total = cnt[0] * n1;                       // <= 2^24: exact as a float
         const float inv1 = 1.0f / (float)n1;
-        for (uint32_t t = lane; t < total && !stop; t += 32) {
+        join_turns(total, [&](uint32_t t) {
           // t / n1 and t mod n1: a float quotient is off by one at most
           uint32_t t0 = (uint32_t)((float)t * inv1);
           int t1 = (int)(t - t0 * n1);
@@ -417,16 +450,16 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
           if (d.sr > 1) {
             const uint32_t c1 = lists[d.row_off[1] + (uint32_t)t1];
             const uint32_t v1 = spread_idx(c1, d.isb[1], d.L);
-            if (((v1 ^ kv) & d.cover[1] & km) != 0u) continue;
+            if (((v1 ^ kv) & d.cover[1] & km) != 0u) return;
             seu &= sea[d.row_off[1] + c1];
-            if (__popc(seu) < 3) continue;
+            if (__popc(seu) < 3) return;
             km |= d.cover[1];
             kv |= v1;
             start = 2;
           }
           if (start == d.sr) {
             if (!emit_lp<kSliding>(d, ldca, rp, kv, z_theta, f, join_local, queue, queue_n)) stop = true;
-            continue;
+            return;
           }
           uint32_t pos[8], skm[8], skv[8], sseu[8];
           int dd = (int)start;
@@ -452,18 +485,10 @@ k_detect(DevParams d, const uint8_t* __restrict__ seav, LdcaRead ldca, const uin
               ++pos[dd];
             }
           }
-        }
+        });
       }
     }
-    __syncwarp();
-    // 3. the warp's LDCA test of the queued complete tuples
-    const uint32_t nq = *queue_n;
-    if (nq >= kTestAt) {
-      test_queue<kSliding>(d, ldca, queue, min(nq, (uint32_t)kHostQueue), z_theta, f, pend, lane);
-      __syncwarp();
-      if (lane == 0) *queue_n = 0;
-    }
-    __syncwarp();
+    __syncwarp();                                      // the lists and the SEA are read
     const bool bound = (__shfl_sync(kFull, ov, 0) & 2u) != 0u;
     stop = __any_sync(kFull, stop) || bound;
     rp = kStaged ? rp_next : next_sea();
