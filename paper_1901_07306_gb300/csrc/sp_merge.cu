@@ -33,17 +33,25 @@ k_zero(uint4* __restrict__ p, uint64_t n16, RouterFlags* __restrict__ flags, uin
 // Routers first .. first + count - 1 of a context: the SEAV, and the LDCA
 // unless bit r of `clean` is set and the router has not spilled.  Every block takes its share
 // of every router (one that is zeroed whole among many skipped ones is spread
-// over the chip).  Blocks read all flags, so the caller clears them after the launch.
+// over the chip), and its warps read the flags of 32 routers at once: a read per
+// router stood before each router's stores.  Blocks read all flags, so the
+// caller clears them after the launch.
 __global__ void __launch_bounds__(kThreads)
 k_reset(uint8_t* __restrict__ base, uint64_t stride, uint64_t seav16, uint32_t first, uint32_t count,
         RouterSet clean, const RouterFlags* __restrict__ flags) {
   const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-  for (uint32_t r = first; r < first + count; ++r) {
-    const bool skip = ((clean.w[r >> 5] >> (r & 31u)) & 1u) != 0u && flags[r].spilled == 0u;
-    uint4* p = reinterpret_cast<uint4*>(base + (uint64_t)r * stride);
-    const uint64_t n16 = skip ? seav16 : stride / 16;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (uint64_t)gridDim.x * blockDim.x)
-      p[i] = z;
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t r0 = first; r0 < first + count; r0 += 32u) {
+    const uint32_t own = r0 + lane;
+    const bool skip = own < first + count && ((clean.w[own >> 5] >> (own & 31u)) & 1u) != 0u && flags[own].spilled == 0u;
+    const uint32_t skips = __ballot_sync(0xFFFFFFFFu, skip);
+    const uint32_t n = min(32u, first + count - r0);
+    for (uint32_t q = 0; q < n; ++q) {
+      uint4* p = reinterpret_cast<uint4*>(base + (uint64_t)(r0 + q) * stride);
+      const uint64_t n16 = ((skips >> q) & 1u) ? seav16 : stride / 16;
+      for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (uint64_t)gridDim.x * blockDim.x)
+        p[i] = z;
+    }
   }
 }
 
