@@ -28,7 +28,7 @@ constexpr uint64_t kBinnedRoundPairs = 1ull << 26;  // pairs per binning round
 // Host-path binning rounds: each round's plane pass overlaps the next round's
 // copies, so after the last copy only one round of 2^24 pairs is left to apply.
 constexpr uint64_t kHostRoundPairs = 1ull << 24;
-constexpr uint32_t kResultPrefix = 2048;            // records fetched with the status (48 KiB)
+constexpr uint32_t kResultPrefix = 4096;            // records fetched with the status, as far as the caller has room (96 KiB)
 // result block: status, error word, batch ticket, `pending` before a binned round, records
 constexpr size_t kKerrAt = 64, kTicketAt = 96, kPriorAt = 100, kRecordsAt = 128;
 constexpr uint32_t kDefaultTimeoutMs = 60000;       // bound of every wait on the stream
