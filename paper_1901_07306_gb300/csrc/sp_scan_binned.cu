@@ -928,8 +928,10 @@ cudaError_t binned_bin_chunk(const DevParams& d, uint8_t* seav, uint32_t* ldca, 
   const uint64_t most = binned_tile_pairs(h) / 2;
   uint64_t quads = 0, full = 0;
   for (uint32_t b = 0; b < src.count; ++b) {
-    quads += src.n[b] / 2;
-    full += src.n[b] / 2 / most;
+    // as k_bin counts them: a first pair off a 16-byte boundary is none of them
+    const uint64_t head = src.n[b] != 0 && ((uintptr_t)src.ptr[b] & 15u) != 0u ? 1u : 0u, q = (src.n[b] - head) / 2;
+    quads += q;
+    full += q / most;
   }
   if (src.count == 1) full = full / s.ctas * s.ctas;
   src.full_max = src.count == 1 ? (uint32_t)full : 0xFFFFFFFFu;
