@@ -32,10 +32,9 @@
 //
 // Staging shapes (the autotuner picks one per context; every shape gives the
 // same bits):  k_bin block size, staging row length, tiles per flush round
-// and blocks per SM -- a 1024-thread block with 44-hip rows flushing every two
-// tiles, or two 512-thread blocks per SM with 20-hip rows flushing every tile,
-// so one block's flush overlaps the other's hashing -- and the k_apply block
-// size.
+// and blocks per SM -- a 1024-thread block with 44-hip rows, or two 512-thread
+// blocks per SM with 20-hip rows, so that one block's flush overlaps the other's
+// hashing; both flush every two of their tiles -- and the k_apply block size.
 #include <cuda.h>
 #include <math.h>
 
@@ -98,11 +97,13 @@ __device__ __forceinline__ void st_chunk(uint32_t* dst, uint4 a, uint4 b) {
 // write-combining buffer for the bin's list).  Per tile:
 //   1. every thread hashes its pairs, queues the sampled pairs (Sec. 3.1) for
 //      a converged SEAV pass, takes a place in its pair's bin row with one
-//      shared atomic and stores the hip there (of a row that is full, which 2 in
-//      a million are by chance, the pair waits for the end of the round: a
-//      single LDCA bit set past the lists would make the fold read 32 MiB of
-//      LDCA, the merge 128 MiB per router of profile D3 and the reset zero them);
-//   2. (after every TPR tiles) each thread takes bins tid, tid + THREADS, ...:
+//      shared atomic and stores the hip there (a pair that finds its row full
+//      waits for the end of the round -- by chance fewer than one in a million
+//      with 44-hip rows, 16 arrivals a round on average, two in a thousand with
+//      20-hip rows and 8 arrivals: a single LDCA bit set past the lists would
+//      make the fold read 32 MiB of LDCA, the merge 128 MiB per router of profile
+//      D3 and the reset zero them);
+//   2. (after every TPR = 2 tiles) each thread takes bins tid, tid + THREADS, ...:
 //      it moves the row's whole 8-hip chunks to the bin's list with 32-byte
 //      stores and keeps the remainder (< 8 hips) at the front of the row; the
 //      queued pairs set their SEAV bits, taken by consecutive threads.
@@ -114,6 +115,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
 k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
       BinSrc src, uint32_t* __restrict__ lists, uint32_t* __restrict__ counts, uint32_t cap,
       bool append, uint32_t rot, RouterFlags* __restrict__ flags, uint32_t* __restrict__ prior) {
+  static_assert(TPR == 2, "one flush round after the tiles of both register buffers");
   constexpr int QUADS = THREADS * kVec;               // 16-byte loads of a whole tile
   constexpr int TILE = QUADS * 2;
   constexpr int QUEUE = TPR * TILE / 32;              // sampled pairs per round: 4x the expected 2^-7
@@ -318,7 +320,7 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
   // Tiles in pairs (i, i + 1) in the two register buffers.  A buffer's loads
   // for tile t + 2 go out as soon as tile t is staged, so the flush round
   // runs with both next tiles in flight (the flush's stores and the stream's
-  // loads overlap); a flush round after every TPR tiles.
+  // loads overlap).
   uint32_t par = 0;
   if (slot < n_tiles) {
     uint4 ra[kVec], rb[kVec];
@@ -327,10 +329,6 @@ k_bin(DevParams d, uint8_t* __restrict__ seav, uint32_t* __restrict__ ldca,
     for (uint32_t t = slot; t < n_tiles; t += 2 * G) {
       stage_tile(ra, par);
       if (t + 2 * G < n_tiles) load_tile(ra, t + 2 * G);
-      if (TPR == 1) {
-        flush_round(par);
-        par ^= 1u;
-      }
       if (t + G < n_tiles) {
         stage_tile(rb, par);
         if (t + 3 * G < n_tiles) load_tile(rb, t + 3 * G);
