@@ -820,7 +820,7 @@ def _serving_runs(S, serve, reqs, total, n_routers, runs, warmup, window_slices)
 def detect_many_leg(torch, sp, n_hosts=150000, reps=50):
     """Detection with many results: n_hosts hosts of 64 distinct peers each at
     theta = 32 (about n_hosts super points, so the result sort spans runs of
-    8,192 keys merged across the grid); detect p50/p99 over reps detects."""
+    2,048 keys merged across the grid); detect p50/p99 over reps detects."""
     rng = np.random.default_rng(51)
     hosts = rng.permutation(np.unique(rng.integers(0, 2**32, n_hosts + n_hosts // 4, dtype=np.uint32))[:n_hosts])
     pairs = np.stack([np.repeat(hosts, 64), rng.integers(0, 2**32, hosts.size * 64, dtype=np.uint32)], 1)

@@ -698,7 +698,7 @@ static int commit_seav_window(sp_ctx* ctx, uint32_t router) {
 // that only binned rounds could have written and that was never folded is
 // still all zero unless its flag says otherwise: a step that merges its
 // routers' planes (sp_merge) never writes their LDCAs, and zeroing the 16 of
-// profile D3 again took 250 of 446 us.  Where that saves nothing (kSkipBytes) one
+// profile D3 again took 325 of 437 us.  Where that saves nothing (kSkipBytes) one
 // plain launch zeroes sketches and flags.
 static int zero_routers(sp_ctx* ctx, uint32_t first, uint32_t count) {
   sp::RouterSet clean{};

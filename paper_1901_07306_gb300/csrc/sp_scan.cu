@@ -338,10 +338,12 @@ int scan_grid(const DevParams& d) {
 
 namespace {
 
-// kHotPairs: at 2^18 pairs of mixed traffic (the heaviest host 1/8 of them)
-// k_scan takes 16.0 us and k_scan_hot 11.9, of uniform traffic 10.9 and 11.9;
-// at 2^17 11.9 both and 7.8 against 11.8.  At 2^20 64 against 26 us (mixed), 26
-// both (uniform).  Two blocks per SM: 3% faster than one from 2^20 on.
+// kHotPairs: kernel times, k_scan and k_scan_hot, us, of mixed traffic (Zipf and
+// planted hosts) 15.9 and 7.9 at 2^18 pairs, 36.5 and 13.5 at 2^19, 52.3 and 22.7
+// at 2^20, 102 and 43.6 at 2^21; of uniform traffic, which has no heavy host, 7.2
+// and 7.4, 12.0 and 13.9, 21.9 and 22.5, 41.7 and 43.6.  At 2^17, with the launch,
+// 11.9 both (mixed) and 7.8 against 11.8 (uniform).  Two blocks per SM: 3% faster
+// than one from 2^20 on.
 template <int LR>
 void scan_launch(const DevParams& d, uint8_t* seav, uint32_t* ldca, const uint32_t* pairs, uint64_t n_pairs,
                  int grid, cudaStream_t s) {

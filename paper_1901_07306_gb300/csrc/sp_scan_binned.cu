@@ -613,7 +613,7 @@ __device__ __forceinline__ void transpose8x4(uint32_t (&x)[8], uint32_t lane) {
 // sources' LDCAs.  One source, the router itself, before a detect, export or
 // copy; the merge of Sec. 4.2 folds all watch points' pending planes at once
 // (16 routers of profile D3: one pass over 16 x 128 MiB of planes instead of 16
-// folds and a merge of 16 LDCAs, 1,668 -> 678 us).
+// folds and a merge of 16 LDCAs, 1,686 -> 443 us).
 // planes: [ceil(W / 8)][k][8] words (W = LR * LC / 32 words per plane, 8-word
 // chunks of the k planes side by side); ldca: [LR * LC][k / 32] words.
 // A source's LDCA is read unless it is null or a flag beside it says that it is
